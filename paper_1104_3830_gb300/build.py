@@ -17,8 +17,9 @@ NVCC_FLAGS = ["-O3", "-std=c++17", "-lineinfo", "-Xcompiler", "-fPIC", "-Xcompil
               "--expt-relaxed-constexpr", "-I", os.path.join(ROOT, "include")]
 
 
-# prune.cu: no FMA contraction, so its keep predicate is bitwise identical everywhere
-PER_FILE_FLAGS = {"prune.cu": ["--fmad=false"]}
+# prune.cu: no FMA contraction, so its keep predicate is bitwise identical everywhere;
+# verify.cu: none either, its products that need one name it
+PER_FILE_FLAGS = {"prune.cu": ["--fmad=false"], "verify.cu": ["--fmad=false"]}
 
 
 def _nvcc() -> str:

@@ -1,6 +1,5 @@
 // prune.cu -- reduced instance B (Eq. matrixred) as CSR, the certificate of Prop. aoc,
-// the LP-duality check of a solution on all of A, FP64 verification of the scaling, and
-// int32 -> int16 narrowing.
+// the LP-duality check of a solution on all of A, and int32 -> int16 narrowing.
 //
 // Keep test: x_ij(p) >= t  <=>  E_ij = p log2 w_ij - U_i - V_j >= log2 t  (log2 units).
 // E is first evaluated in FP32 with the same centring as the sweeps; when it lies within
@@ -269,50 +268,6 @@ __global__ void to_f32_kernel(const double* x, float* y, int n) {
     if (k < n) y[k] = (float)x[k];
 }
 
-// ---- FP64 verification of row / column sums -----------------------------------------
-__global__ void verify_rows_kernel(const void* w, int i16, int n, int64_t ld, double p,
-                                   const double* u, const double* v, double* rows, double* err) {
-    const int i = blockIdx.x;
-    double s = 0.0;
-    for (int j = threadIdx.x; j < n; j += blockDim.x) {
-        const int wv = i16 ? (int)((const int16_t*)w)[(int64_t)i * ld + j] : ((const int32_t*)w)[(int64_t)i * ld + j];
-        if (wv > 0) s += exp(p * log((double)wv) - u[i] - v[j]);
-    }
-    s = warp_sum(s);
-    __shared__ double sh[32];
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = s;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t += sh[k];
-        if (rows) rows[i] = t;
-        err[i] = fabs(t - 1.0);
-    }
-}
-
-__global__ void verify_cols_kernel(const void* w, int i16, int n, int64_t ld, double p,
-                                   const double* u, const double* v, int rows_per_chunk,
-                                   double* part) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    const int r0 = blockIdx.y * rows_per_chunk, r1 = min(n, r0 + rows_per_chunk);
-    double s = 0.0;
-    for (int i = r0; i < r1; ++i) {
-        const int wv = i16 ? (int)((const int16_t*)w)[(int64_t)i * ld + j] : ((const int32_t*)w)[(int64_t)i * ld + j];
-        if (wv > 0) s += exp(p * log((double)wv) - u[i] - v[j]);
-    }
-    part[(int64_t)blockIdx.y * n + j] = s;
-}
-
-__global__ void verify_cols_combine(int n, int nchunks, const double* part, double* cols, double* err) {
-    const int j = blockIdx.x * blockDim.x + threadIdx.x;
-    if (j >= n) return;
-    double s = 0.0;
-    for (int c = 0; c < nchunks; ++c) s += part[(int64_t)c * n + j];
-    if (cols) cols[j] = s;
-    err[j] = fabs(s - 1.0);
-}
-
 // smallest positive and largest weight of the matrix (zeros are absent entries)
 __global__ void minmax_kernel(const void* w, int i16, int n, int64_t ld, unsigned long long* out) {
     unsigned mn = 0xffffffffu, mx = 0u;
@@ -332,20 +287,6 @@ __global__ void minmax_kernel(const void* w, int i16, int n, int64_t ld, unsigne
     if ((threadIdx.x & 31) == 0) {
         atomicMin(out, (unsigned long long)mn);
         atomicMax(out + 1, (unsigned long long)mx);
-    }
-}
-
-__global__ void max_reduce_kernel(const double* x, int n, double* out) {
-    double m = 0.0;
-    for (int k = threadIdx.x; k < n; k += blockDim.x) m = fmax(m, x[k]);
-    m = warp_max(m);
-    __shared__ double sh[32];
-    if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        double t = 0.0;
-        for (int k = 0; k < (int)(blockDim.x >> 5); ++k) t = fmax(t, sh[k]);
-        *out = t;
     }
 }
 
@@ -510,42 +451,6 @@ sa_status certify_device(sa_ctx* ctx, const sa_matrix* a, const double* alpha, c
             add->w[x] = hw[order[x]];
         }
     }
-    return SA_OK;
-}
-
-sa_status verify_device(sa_ctx* ctx, const sa_matrix* a, double p, const double* d_u,
-                        const double* d_v, double* d_rows, double* d_cols, double* max_row_err,
-                        double* max_col_err) {
-    const int n = a->n;
-    cudaStream_t st = ctx->stream;
-    const int rows_per_chunk = 256;
-    const int nchunks = (n + rows_per_chunk - 1) / rows_per_chunk;
-    size_t need = 2 * align_up((size_t)n * 8, 256) + align_up((size_t)nchunks * n * 8, 256) + 4096;
-    sa_status rc = ctx->ws.reserve(need);
-    if (rc) return rc;
-    Carve cv(ctx->ws.ptr);
-    double* rerr = cv.take<double>(n);
-    double* cerr = cv.take<double>(n);
-    double* part = cv.take<double>((size_t)nchunks * n);
-    double* mx = cv.take<double>(2);
-    const int i16 = a->wtype == SA_I16;
-    verify_rows_kernel<<<n, 256, 0, st>>>(a->w, i16, n, a->ld, p, d_u, d_v, d_rows, rerr);
-    count_launch();
-    dim3 g((n + 127) / 128, nchunks);
-    verify_cols_kernel<<<g, 128, 0, st>>>(a->w, i16, n, a->ld, p, d_u, d_v, rows_per_chunk, part);
-    count_launch();
-    verify_cols_combine<<<(n + 255) / 256, 256, 0, st>>>(n, nchunks, part, d_cols, cerr);
-    count_launch();
-    max_reduce_kernel<<<1, 1024, 0, st>>>(rerr, n, mx);
-    count_launch();
-    max_reduce_kernel<<<1, 1024, 0, st>>>(cerr, n, mx + 1);
-    count_launch();
-    double h[2];
-    SA_CUDA(cudaMemcpyAsync(h, mx, 16, cudaMemcpyDeviceToHost, st));
-    SA_CUDA(cudaStreamSynchronize(st));
-    SA_CUDA(cudaGetLastError());
-    if (max_row_err) *max_row_err = h[0];
-    if (max_col_err) *max_col_err = h[1];
     return SA_OK;
 }
 

@@ -171,7 +171,7 @@ void launch_scale_vec(double* x, int n, double f, cudaStream_t s);
 // Vh = float(V), Vc = 2^(Vh - V)
 void launch_split_v(const double* V, float* Vh, float* Vc, int n, cudaStream_t s);
 
-// ---- prune / certify / verify (prune.cu) --------------------------------------------
+// ---- prune and certify (prune.cu), verify (verify.cu) ---------------------------------
 sa_status prune_device(sa_ctx* ctx, const sa_matrix* a, double p, const double* d_u,
                        const double* d_v, double t, int guard, sa_csr* out, double* log_ub);
 sa_status certify_device(sa_ctx* ctx, const sa_matrix* a, const double* alpha,
