@@ -122,3 +122,55 @@ def test_narrowing(ctx):
     assert np.array_equal(dst.cpu().numpy().astype(np.int32), w)
     src[3, 4] = 40000
     assert api.sa_narrow_i32_to_i16(ctx, src, dst) == 1
+
+
+@pytest.mark.parametrize("n,dtype,hi,padded,zeros", [(1, np.int16, 9, True, False), (7, np.int32, 50, False, True),
+                                                     (255, np.int16, 1000, True, True), (256, np.int32, 1000, True, False),
+                                                     (257, np.int16, 1000, False, True), (1030, np.int32, 2 ** 30, True, True),
+                                                     (1100, np.int16, 4, True, True)])
+@pytest.mark.parametrize("guard", [True, False])
+def test_prune_and_certify_edges(ctx, n, dtype, hi, padded, zeros, guard):
+    """Edges of the scans' tiles (256 columns, 32 x 32 keep bits, up to 256 rows a block), rows
+    off 16-byte boundaries, absent entries and many equal weights (the guards' lowest index)."""
+    rng = np.random.default_rng(n)
+    w = rng.integers(1, hi + 1, (n, n)).astype(dtype)
+    if zeros:
+        w[rng.random((n, n)) < 0.3] = 0
+        w[np.arange(n), np.arange(n)] = 1
+    p = 4.0
+    b = oracle.log_weights(w.astype(np.int64))
+    # potentials with all but three bits of their mantissa zero, so that equal weights of equal
+    # columns tie exactly in FP32 as in FP64
+    u = np.round(p * np.log(max(hi, 2)) * 4) / 4 + rng.integers(-3, 4, n) * 0.25
+    v = rng.integers(-2, 3, n) * 0.25
+    d = api.to_device(w) if padded else torch.from_numpy(w).cuda()
+    rp, col, wv, ub = api.sa_prune(ctx, d, p, torch.from_numpy(u).cuda(), torch.from_numpy(v).cuda(), 0.0, guard)
+    rows = np.repeat(np.arange(n), np.diff(rp))
+    assert rp[0] == 0 and rp[-1] == len(col) and np.array_equal(wv, w[rows, col])
+    for i in range(n):
+        assert np.all(np.diff(col[rp[i]:rp[i + 1]]) > 0)
+    got = np.zeros((n, n), dtype=bool)
+    got[rows, col] = True
+    e = p * b - u[:, None] - v[None, :]
+    above = e >= np.log(1.0 / n)
+    near = np.abs(e - np.log(1.0 / n)) < 1e-9
+    assert np.array_equal((got & above) & ~near, above & ~near)
+    extra = got & ~above & ~near
+    if guard:   # beyond the threshold only row and column maxima, one a row and column
+        m = (e >= e.max(1, keepdims=True) - 2e-4) | (e >= e.max(0, keepdims=True) - 2e-4)
+        assert not np.any(extra & ~m) and extra.sum() <= 2 * n
+        assert got.any(1).all() and got.any(0).all()
+    else:
+        assert not extra.any()
+    assert abs(ub - oracle.log_ub(b, p, v)) < 1e-9 * max(1.0, abs(ub)) + 1e-4 * n / p
+    # duals on the row maxima but for a few rows
+    beta = v / p
+    alpha = (b - beta).max(1)
+    alpha[::3] -= 0.37
+    nv, (arp, acol, aw) = api.sa_certify(ctx, d, alpha, beta, 1e-9, max_add=n * n)
+    viol = b - alpha[:, None] - beta > 1e-9
+    assert nv == viol.sum() == arp[-1]
+    got = np.zeros((n, n), dtype=bool)
+    ar = np.repeat(np.arange(n), np.diff(arp))
+    got[ar, acol] = True
+    assert np.array_equal(got, viol) and np.array_equal(aw, w[ar, acol])
