@@ -72,8 +72,9 @@ typedef enum { SA_PREC_MIXED = 0, SA_PREC_FP32 = 1, SA_PREC_FP64 = 2 } sa_prec;
  *   2^-40, one SFU exp2) into a workspace of n * ceil(n/4)*4 floats, and each sweep reads K once
  *   (4 bytes per element): no per-element SFU work in the sweeps and an error that does
  *   not grow with p.  The first evaluation of a call also keeps log2 w as a float pair
- *   (8 bytes per element), which the later ones read instead of the weights.  Needs
- *   n <= 24576 (above 12288 the shared-memory ring holds one row per stage).
+ *   (8 bytes per element), which the later ones read instead of the weights.  Where K fits
+ *   in the registers and shared memory of the grid (n up to about 3300 on a whole GB300),
+ *   the sweeps keep it there.  Needs n <= 24576 (above 12288 the shared-memory ring holds one row per stage).
  * NEWTON: the Newton variant of Sec. 5.3 (Knight-Ruiz iteration on the symmetric
  *   embedding S = [[0, A], [A^T, 0]], conjugate gradients for each Newton system).  At
  *   every p step it evaluates the same K as STEP, then iterates on K; each CG iteration

@@ -450,6 +450,8 @@ sa_status sa_scale(sa_ctx* ctx, const sa_matrix* a, const sa_scale_opts* o, doub
         return SA_E_UNSUPPORTED;
     }
     NvtxRange range("sa_scale n=%d kernel=%d p_steps=%d", n, (int)kind, o->n_p);
+    // the STEP path where K fits on the chip: its potentials come back in natural units
+    const bool natural = kind == SA_KERNEL_STEP && resident_supported(ctx, a, o);
     // library units: log2.  A warm start is kept so that a failure leaves the caller's
     // potentials as they were given.
     if (o->resume_from > 0) {
@@ -461,10 +463,12 @@ sa_status sa_scale(sa_ctx* ctx, const sa_matrix* a, const sa_scale_opts* o, doub
         launch_scale_vec(d_v, n, kLog2e, ctx->stream);
     }
     if (kind == SA_KERNEL_NEWTON) rc = scale_newton(ctx, a, o, d_u, d_v, info);
+    else if (natural) rc = scale_resident(ctx, a, o, d_u, d_v, info);
     else if (kind == SA_KERNEL_STEP) rc = scale_step(ctx, a, o, d_u, d_v, info);
     else if (kind == SA_KERNEL_FUSED) rc = scale_fused(ctx, a, o, d_u, d_v, info);
     else rc = scale_plain(ctx, a, o, d_u, d_v, info);
     if (rc == SA_OK || rc == SA_E_NOT_CONVERGED) {
+        if (natural) return rc;
         launch_scale_vec(d_u, n, kLn2, ctx->stream);
         launch_scale_vec(d_v, n, kLn2, ctx->stream);
         cudaError_t e = cudaStreamSynchronize(ctx->stream);

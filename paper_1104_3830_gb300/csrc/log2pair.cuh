@@ -58,4 +58,19 @@ __device__ __forceinline__ float2 wlog2(const float4* stab, int w) {
     return make_float2(hi, (float)(l - (double)hi));
 }
 
+// 2^(p log2 w - V_j - m) with the operands as float pairs (p = ph + pl): the large leading
+// parts cancel exactly (two-product, two-sums), the small ones are added after; the exponent
+// x is then exact to about 2^-24 |x|
+__device__ __forceinline__ float pair_exp2(float ph, float pl, float2 lw, float vh, float vl, float mh, float ml) {
+    const float t = ph * lw.x;
+    const float te = fmaf(ph, lw.x, -t);
+    float e1, e2;
+    const float s1 = two_sum(t, -vh, &e1);
+    const float s2 = two_sum(s1, -mh, &e2);
+    const float rest = ((te + e1) + e2) + (fmaf(ph, lw.y, pl * lw.x) - vl - ml);
+    float y;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(s2 + rest));
+    return y;
+}
+
 }  // namespace sa

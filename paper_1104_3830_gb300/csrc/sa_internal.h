@@ -160,6 +160,10 @@ bool fused_supported(const sa_ctx* ctx, const sa_matrix* a);
 sa_status scale_step(sa_ctx* ctx, const sa_matrix* a, const sa_scale_opts* o, double* U,
                      double* V, sa_scale_info* info);
 bool step_supported(const sa_ctx* ctx, const sa_matrix* a);
+// sweep_resident.cu: the same on a K that stays on the chip; potentials come back in natural units
+sa_status scale_resident(sa_ctx* ctx, const sa_matrix* a, const sa_scale_opts* o, double* U,
+                         double* V, sa_scale_info* info);
+bool resident_supported(const sa_ctx* ctx, const sa_matrix* a, const sa_scale_opts* o);
 size_t fused_workspace_bytes(const sa_ctx* ctx, const sa_matrix* a);
 // newton.cu: Newton scaling of Sec. 5.3 on the per-step matrix (SA_KERNEL_NEWTON)
 sa_status scale_newton(sa_ctx* ctx, const sa_matrix* a, const sa_scale_opts* o, double* U,

@@ -465,18 +465,7 @@ __global__ void __launch_bounds__(NT, 1) step_kernel(StepArgs A) {
 #pragma unroll
                 for (int e = 0; e < 4; ++e) {
                     if (lh[e] > -INFINITY) {
-                        // x = p log2 w - V_j - m with 48-bit operands: the large leading
-                        // parts cancel exactly (two-product, two-sums), the small ones are
-                        // added after; x is then exact to about 2^-24 |x|
-                        const float2 lw = make_float2(lh[e], ll[e]);
-                        const float2 vj = make_float2(vh[e], vl[e]);
-                        const float t = ph * lw.x;
-                        const float te = fmaf(ph, lw.x, -t);
-                        float e1, e2;
-                        const float s1 = two_sum(t, -vj.x, &e1);
-                        const float s2 = two_sum(s1, -mh, &e2);
-                        const float rest = ((te + e1) + e2) + (fmaf(ph, lw.y, pl * lw.x) - vj.y - ml);
-                        kv[e] = ex2_approx(s2 + rest);
+                        kv[e] = pair_exp2(ph, pl, make_float2(lh[e], ll[e]), vh[e], vl[e], mh, ml);
                     }
                 }
                 if (cidx[k] < NC) *(float4*)(krow + cidx[k] * 4) = make_float4(kv[0], kv[1], kv[2], kv[3]);

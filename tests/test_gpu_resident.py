@@ -1,0 +1,95 @@
+"""The step kernel on a K that stays on the chip (matrices up to n of about 3300) at the edges of
+its shapes.  Tolerances are the step path's (test_gpu_step): both sides stop within
+tol = 1e-6 of bistochastic, so X agrees with the oracle's to 8e-6 max(x, 1/n) and its FP64 sums
+are within tol + 1e-6 of one."""
+import numpy as np
+import pytest
+
+import oracle
+from paper_1104_3830_gb300 import api
+from paper_1104_3830_gb300 import workloads as W
+
+torch = pytest.importorskip("torch")
+pytestmark = pytest.mark.gpu
+
+SUM_BOUND = 2e-6
+
+
+@pytest.fixture(scope="module")
+def ctx():
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    from paper_1104_3830_gb300 import build
+    build.build()
+    c = api.sa_create(0)
+    yield c
+    c.close()
+
+
+def _check(ctx, w, d, ps, u, v, info, against_oracle):
+    assert info["status"] == 0 and info["kernel_used"] == 3, info
+    assert max(api.sa_verify(ctx, d, ps[-1], u, v)) < SUM_BOUND
+    if against_oracle:
+        b = oracle.log_weights(w.astype(np.int64))
+        uo, vo, _, _, st = oracle.sinkhorn(b, ps, 1e-6, 20000)
+        assert st == 0
+        x, xo = (oracle.xmatrix(b, ps[-1], *uv) for uv in ((u.cpu().numpy(), v.cpu().numpy()), (uo, vo)))
+        assert np.all(np.abs(x - xo) <= 8e-6 * np.maximum(xo, 1.0 / w.shape[0]) + 1e-9)
+
+
+# one row, one block and several, the edges of the widths (512, 1024, 2048 columns of threads),
+# of the rows in registers (8 a block up to n = 1216, 14 up to 2048) and near the largest that fit
+@pytest.mark.parametrize("n", [1, 5, 16, 71, 511, 513, 1001, 1216, 1217, 2047, 2050, 3333])
+@pytest.mark.parametrize("dtype", [np.int16, np.int32])
+def test_resident_shapes(ctx, n, dtype):
+    w = W.uniform(n, 1, 30000 if dtype == np.int16 else 1 << 20, 40 + n, dtype=dtype)
+    if n > 16:   # absent entries and columns of very different mass
+        w[:: 3, 1:: 7] = 0
+        w[:, n // 2:] = np.maximum(w[:, n // 2:] >> 6, (w[:, n // 2:] > 0).astype(dtype))
+    d = api.to_device(w)
+    ps = [1.0, 2.0, 4.0, 8.0]
+    u, v, info = api.sa_scale(ctx, d, ps, 1e-6, 20000, kernel="step")
+    _check(ctx, w, d, ps, u, v, info, n <= 1217)
+
+
+@pytest.mark.parametrize("grid", [1, 8, 20, 76])
+def test_resident_capped_grids(ctx, grid):
+    """Longer stripes on fewer blocks (and the streaming kernel where they do not fit)."""
+    n = 300
+    w = W.uniform(n, 1, 1000, 43, dtype=np.int16)
+    d = api.to_device(w)
+    ps = [1.0, 4.0]
+    api.sa_set_option(ctx, "max_grid", grid)
+    try:
+        u, v, info = api.sa_scale(ctx, d, ps, 1e-6, 20000, kernel="step")
+    finally:
+        api.sa_set_option(ctx, "max_grid", 0)
+    _check(ctx, w, d, ps, u, v, info, True)
+
+
+def test_resident_resume_keep_and_large_steps(ctx):
+    n = 700
+    w = W.uniform(n, 1, 1000, 41, dtype=np.int16)
+    d = api.to_device(w)
+    ps = [1.0, 2.0, 4.0, 8.0, 16.0]
+    u, v, _ = api.sa_scale(ctx, d, ps[:3], 1e-6, 20000, kernel="step")
+    u, v, info = api.sa_scale(ctx, d, ps, 1e-6, 20000, kernel="step", resume_from=3, u=u, v=v)
+    assert info["steps_done"] == 2
+    _check(ctx, w, d, ps, u, v, info, True)
+    kept = [1.0, 1.25, 1.5]
+    u, v, info = api.sa_scale(ctx, d, kept, 1e-6, 20000, kernel="step", warm_keep_v=True)
+    _check(ctx, w, d, kept, u, v, info, True)
+    # p times 64: references from the row maxima, not from the scaled potentials
+    u, v, info = api.sa_scale(ctx, d, [1.0, 64.0], 1e-6, 20000, kernel="step")
+    _check(ctx, w, d, [1.0, 64.0], u, v, info, False)
+
+
+@pytest.mark.parametrize("steps,cap", [(64, 100), (65, 100), (2, 1 << 30)])
+def test_resident_limits(ctx, steps, cap):
+    """The longest schedule it takes, and calls beyond its parameters (the streaming kernel)."""
+    w = W.uniform(100, 1, 1000, 42, dtype=np.int32)
+    d = api.to_device(w)
+    ps = [1.0 + 0.05 * k for k in range(steps)]
+    u, v, info = api.sa_scale(ctx, d, ps, 1e-6, cap, kernel="step")
+    assert info["steps_done"] == steps
+    _check(ctx, w, d, ps, u, v, info, True)
