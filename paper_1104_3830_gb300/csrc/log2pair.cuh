@@ -5,7 +5,14 @@
 #include <cuda_runtime.h>
 #include <math.h>
 
+#include "sa_internal.h"
+
 namespace sa {
+
+// Row references of K from scaled row potentials lie up to cs log2 n above the row maxima (cs:
+// the ratio of the p values); beyond this many powers of two the maxima are taken instead,
+// while the largest entries of K are still far above the FP32 underflow.
+constexpr double kMaxRefShift = 64.0;
 
 constexpr int kLog2Tab = 32768;   // weights below this take the shared-table logarithm
 
@@ -71,6 +78,26 @@ __device__ __forceinline__ float pair_exp2(float ph, float pl, float2 lw, float 
     float y;
     asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(s2 + rest));
     return y;
+}
+
+// log2 of s > 0 in FP64: the mantissa times a 9-bit reciprocal from the table is 1 + r exactly,
+// |r| < 2^-7; near 1 r = s - 1 itself.  ltab[j] = -log2(tab[j].x) in FP64.  One formula for all
+// arguments, about 20 FP64 instructions where the library's log2 takes some hundred: GB300 runs
+// two of them per clock and SM.
+__device__ __forceinline__ double sum_log2(double s, const float4* tab, const double* ltab) {
+    const int hi = __double2hiint(s);
+    const int e = (hi >> 20) - 1023;
+    const int idx = (hi >> 12) & 255;
+    const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(s));
+    const double d = s - 1.0;
+    const bool near = fabs(d) < 0x1p-8;
+    const double r = near ? d : fma(m, (double)tab[idx].x, -1.0);
+    const double base = near ? 0.0 : (double)e + ltab[idx];
+    // ln(1 + r) / r up to r^6 (the next term is below 2^-59)
+    const double r2 = r * r;
+    const double a = fma(r, -0.5, 1.0), b = fma(r, -0.25, 1.0 / 3.0), c = fma(r, -1.0 / 6.0, 0.2);
+    const double q = fma(r2, fma(r2, fma(r2, 1.0 / 7.0, c), b), a);
+    return fma(r * kLog2e, q, base);
 }
 
 }  // namespace sa

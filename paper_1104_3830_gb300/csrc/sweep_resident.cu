@@ -38,7 +38,6 @@ namespace {
 
 constexpr int kResMaxP = 64;       // p steps of a call (the schedule is a kernel parameter)
 constexpr int kResMaxRows = 32;    // rows (and columns) of a block
-constexpr double kResMaxShift = 64.0;
 // Copies of the column factors, each polled by its share of the blocks: with one copy the
 // polls of 150 blocks queued at the few L2 lines that hold the factors and kept the owners'
 // stores waiting (7000 to 9000 cycles from a store to its last reader at n = 1200 .. 2047).
@@ -144,25 +143,6 @@ __device__ __forceinline__ unsigned float_key(float x) {
 }
 __device__ __forceinline__ float key_float(unsigned k) {
     return __uint_as_float((k & 0x80000000u) ? (k & 0x7fffffffu) : ~k);
-}
-
-// log2 of s > 0 in FP64: the mantissa times a 9-bit reciprocal from the table is 1 + r exactly,
-// |r| < 2^-8; near 1 r = s - 1 itself.  One formula for all sums, so that the lanes of a warp do
-// not part (the library's log2 took 2 us of a sweep wherever a sum was 1e-3 or more from 1).
-__device__ __forceinline__ double sum_log2(double s, const float4* tab, const double* ltab) {
-    const int hi = __double2hiint(s);
-    const int e = (hi >> 20) - 1023;
-    const int idx = (hi >> 12) & 255;
-    const double m = __hiloint2double((hi & 0xfffff) | 0x3ff00000, __double2loint(s));
-    const double d = s - 1.0;
-    const bool near = fabs(d) < 0x1p-8;
-    const double r = near ? d : fma(m, (double)tab[idx].x, -1.0);
-    const double base = near ? 0.0 : (double)e + ltab[idx];
-    // ln(1 + r) / r up to r^6 (the next term is below 2^-59)
-    const double r2 = r * r;
-    const double a = fma(r, -0.5, 1.0), b = fma(r, -0.25, 1.0 / 3.0), c = fma(r, -1.0 / 6.0, 0.2);
-    const double q = fma(r2, fma(r2, fma(r2, 1.0 / 7.0, c), b), a);
-    return fma(r * kLog2e, q, base);
 }
 
 // four weights of row `row` from column j (cnt of them in the matrix, zeros after)
@@ -370,7 +350,7 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
             // the scaled row potentials lie within cs log2 n above the row maxima: references as
             // long as the largest entry of a row stays far above the FP32 underflow, else the maxima
             double cs = k > 0 && !A.keep_v ? p / A.P[k - 1] : 0.0;
-            if (cs * (double)(32 - __clz(n)) > kResMaxShift) cs = 0.0;
+            if (cs * (double)(32 - __clz(n)) > kMaxRefShift) cs = 0.0;
             const float pf = (float)p, ph = pf, pl = (float)(p - (double)ph);
             float vh[M], vl[M];
 #pragma unroll

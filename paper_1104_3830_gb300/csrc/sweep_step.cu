@@ -551,7 +551,9 @@ __global__ void __launch_bounds__(NT, 1) step_kernel(StepArgs A) {
             // the first evaluation of a step after a step (or a resumed one) scaled (u, v):
             // row references from U; otherwise the row maxima
             {
-                const double cs = (k > 0 && !A.keep_v && step_reanchors == 0) ? p / A.P[k - 1] : 0.0;
+                double cs = (k > 0 && !A.keep_v && step_reanchors == 0) ? p / A.P[k - 1] : 0.0;
+                // far steps of p: the maxima as well, K would underflow below them
+                if (cs * (double)(32 - __clz(n)) > kMaxRefShift) cs = 0.0;
                 if (l_ready) {
                     prep(p, cs, std::false_type{});
                 } else {
@@ -684,7 +686,8 @@ __global__ void __launch_bounds__(NT, 1) step_kernel(StepArgs A) {
                         if (r < nr && !(ss[r] >= 0x1p-120f && ss[r] <= 0x1p120f)) ss_bad = true;
                     }
                     if (ss_bad) {
-                        if (tid == 0) atomicCAS(A.err, 0, kErrNonfinite);
+                        // every thread: thread 0 may leave the pass on another's flag before it gets here
+                        atomicCAS(A.err, 0, kErrNonfinite);
                         s_flag = 1;
                         return false;
                     }

@@ -270,3 +270,17 @@ def test_sparse_epochs_match_dense(ctx, n):
     assert np.max(np.abs(xs - xd)) < tol_x, np.max(np.abs(xs - xd))
     # the planted permutation carries the mass at p = 512
     assert np.all(xs[np.arange(n), pi] > 0.5)
+
+
+def test_far_steps_of_p(ctx):
+    """p times 64 and times 256 in one step (n = 4000, K streamed): the scaled potentials lie
+    hundreds of powers of two above the row maxima, the references come from the maxima."""
+    w = W.uniform(4000, 1, 1000, 950, dtype=np.int16)
+    d = api.to_device(w)
+    u, v, info = api.sa_scale(ctx, d, [1.0, 64.0], 1e-6, 20000, kernel="step")
+    assert info["status"] == 0 and info["steps_done"] == 2, info
+    assert max(api.sa_verify(ctx, d, 64.0, u, v)) < STEP_SUM_BOUND
+    u, v, info = api.sa_scale(ctx, d, [1.0, 256.0], 1e-12, 3, kernel="step")
+    assert info["status"] == -4 and info["sweeps_total"] == 6, info
+    er, ec = api.sa_verify(ctx, d, 256.0, u, v)
+    assert ec < 1e-5 and np.isfinite(er)
