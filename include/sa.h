@@ -444,10 +444,10 @@ sa_status sa_narrow_i32_to_i16(sa_ctx* ctx, const int32_t* d_src, int64_t ld_src
  * REGS: as GROUP, with K in registers during the sweeps (each row and column of K split
  *   over 32 G / NMAX adjacent lanes): 1, 2 or 4 warps for n <= 32, 4 or 8 for n <= 64, 16
  *   for n <= 128.
- * KROWS: one block of 256 threads per instance (n <= 512) on the same K, kept in a global
- *   slot of n x ceil(n/4)*4 FP32 per block (taken from the context workspace: up to two
- *   blocks per SM); each warp evaluates and reads whole rows, so a row sum needs no block
- *   barrier, and a sweep has one; the error does not grow with p. */
+ * KROWS: n <= 512 on the same K, held in registers and shared memory by one thread block
+ *   (n <= 144) or by a cluster of two or four; a global slot per cluster (taken from the
+ *   context workspace) keeps log2 w as float pairs between the p steps; the error does not
+ *   grow with p. */
 typedef enum { SA_BATCH_BLOCK = 0, SA_BATCH_GROUP = 1, SA_BATCH_REGS = 2, SA_BATCH_KROWS = 3 } sa_batch_path;
 
 /* A launch plan: instances are grouped by n into buckets (n_hi[b-1], n_hi[b]] (n_hi

@@ -21,8 +21,8 @@
 #include <numeric>
 #include <vector>
 
+#include "batch_cluster.cuh"
 #include "common.cuh"
-#include "krows.cuh"
 #include "log2pair.cuh"
 #include "sa_internal.h"
 
@@ -49,8 +49,8 @@ struct BatchArgs {
     int32_t* status;        // per instance: 0 ok, 1 not converged, -6 nonfinite
     unsigned* queue;        // work counter
     size_t smem_table;      // bytes available for the log2 table
-    float* kscr;            // K rows path: a global slot of K per block
-    size_t kscr_floats;     // floats of one block's slot
+    float* kscr;            // K rows path: a global slot per cluster (the staging of K, log2 w pairs)
+    size_t kscr_floats;     // floats of one cluster's slot
 };
 
 template <typename WT, int NT, int KC>
@@ -735,26 +735,12 @@ __global__ void __launch_bounds__(512) batch_regs_kernel(BatchArgs A) {
 }
 
 // ---------------------------------------------------------------------------------------
-// K rows path: the larger instances (n <= 128 CH) one per block of 256 threads (krows.cuh),
-// each block on a global-memory slot of K of its own.
+// K rows path (batch_cluster.cuh): an instance on a block, or on a cluster of two or four, that holds its
+// K on the chip; kscr holds a slot of three n x ceil(n/4)*4 planes per cluster.
 // ---------------------------------------------------------------------------------------
-template <typename WT, int CH>
-__global__ void __launch_bounds__(256, 2) batch_krows_kernel(BatchArgs A) {
-    __shared__ KrowsSmem<CH> sm;
-    __shared__ int s_inst;
-    krows_init(sm);
-    float* K = A.kscr + (size_t)blockIdx.x * A.kscr_floats;
-    for (;;) {
-        if (threadIdx.x == 0) {
-            const unsigned q = atomicAdd(A.queue, 1u);
-            s_inst = q < (unsigned)A.k ? A.order[q] : -1;
-        }
-        __syncthreads();
-        const int inst = s_inst;
-        if (inst < 0) break;
-        krows_instance<WT, CH>(sm, (const WT*)A.w[inst], A.n[inst], A.ld[inst], A.P, A.n_p, A.tol, A.max_sweeps, K,
-                               A.U + A.off[inst], A.V + A.off[inst], A.sweeps + inst, A.status + inst);
-    }
+template <typename WT, int NT, int C, int CH, int RG, int RS>
+__global__ void __launch_bounds__(NT, 512 / NT) batch_cluster_kernel(BatchArgs A) {
+    cluster_instances<WT, NT, C, CH, RG, RS>(A, A.kscr + (size_t)(blockIdx.x / C) * A.kscr_floats);
 }
 
 }  // namespace
@@ -857,24 +843,68 @@ sa_status launch_group_path(sa_ctx* ctx, cudaStream_t bs, const BatchArgs& args,
     return launch_group_n<int32_t, 4>(ctx, bs, args, nmax, per_block);
 }
 
-// K rows path: one block of 256 threads per instance, two blocks per SM, a global slot of
-// K per block (args.kscr, args.kscr_floats); `blocks` is the grid the slots were sized for
-sa_status launch_krows_path(sa_ctx* ctx, cudaStream_t bs, const BatchArgs& args, int nmax, int blocks,
-                            sa_wtype wtype) {
-    auto go = [&](auto kern) -> sa_status {
-        kern<<<blocks, 256, 0, bs>>>(args);
-        count_launch();
-        SA_CUDA(cudaGetLastError());
+// K rows path: blocks and threads of an instance by its n (the fewest that hold K; half an SM
+// each up to 256, so that two instances overlap their reductions, a whole one above, where the
+// exchange between more blocks costs more than the overlap gives).
+constexpr int kClusterHi[4] = {144, 256, 384, 512};
+inline int cluster_class(int n) { return n <= kClusterHi[0] ? 0 : n <= kClusterHi[1] ? 1 : n <= kClusterHi[2] ? 2 : 3; }
+inline int cluster_blocks(int cls) { return cls == 0 ? 1 : cls == 3 ? 4 : 2; }
+inline int cluster_threads(int cls) { return cls < 2 ? 256 : 512; }
+
+template <typename WT, int NT, int C, int CH, int RG, int RS, typename F>
+sa_status one_cluster_kernel(F&& f) {
+    return f(batch_cluster_kernel<WT, NT, C, CH, RG, RS>, sizeof(ClusterSmem<NT, C, CH, RG, RS>));
+}
+template <typename WT, typename F>
+sa_status cluster_kernel_of(int cls, F&& f) {
+    if (cls == 0) return one_cluster_kernel<WT, 256, 1, 2, 6, 12>(f);
+    if (cls == 1) return one_cluster_kernel<WT, 256, 2, 2, 6, 10>(f);
+    if (cls == 2) return one_cluster_kernel<WT, 512, 2, 3, 4, 8>(f);
+    return one_cluster_kernel<WT, 512, 4, 4, 4, 4>(f);
+}
+template <typename F>
+sa_status with_cluster_kernel(int cls, sa_wtype wtype, F&& f) {
+    return wtype == SA_I16 ? cluster_kernel_of<int16_t>(cls, f) : cluster_kernel_of<int32_t>(cls, f);
+}
+
+// Clusters of the class that run at once (0: the kernel does not fit), into *count.
+sa_status cluster_capacity(sa_ctx* ctx, int cls, sa_wtype wtype, int* count) {
+    return with_cluster_kernel(cls, wtype, [&](auto kern, size_t smem) -> sa_status {
+        const int C = cluster_blocks(cls);
+        SA_CUDA(allow_dynamic_smem(kern, ctx->smem_optin));
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(2 * ctx->num_sms / C * C);
+        cfg.blockDim = dim3(cluster_threads(cls));
+        cfg.dynamicSmemBytes = smem;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = C;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        SA_CUDA(cudaOccupancyMaxActiveClusters(count, kern, &cfg));
         return SA_OK;
-    };
-    if (wtype == SA_I16) {
-        if (nmax <= 128) return go(batch_krows_kernel<int16_t, 1>);
-        if (nmax <= 256) return go(batch_krows_kernel<int16_t, 2>);
-        return go(batch_krows_kernel<int16_t, 4>);
-    }
-    if (nmax <= 128) return go(batch_krows_kernel<int32_t, 1>);
-    if (nmax <= 256) return go(batch_krows_kernel<int32_t, 2>);
-    return go(batch_krows_kernel<int32_t, 4>);
+    });
+}
+
+sa_status launch_cluster_path(cudaStream_t bs, const BatchArgs& args, int cls, int clusters, sa_wtype wtype) {
+    return with_cluster_kernel(cls, wtype, [&](auto kern, size_t smem) -> sa_status {
+        const int C = cluster_blocks(cls);
+        cudaLaunchConfig_t cfg{};
+        cfg.gridDim = dim3(clusters * C);
+        cfg.blockDim = dim3(cluster_threads(cls));
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = bs;
+        cudaLaunchAttribute at[1];
+        at[0].id = cudaLaunchAttributeClusterDimension;
+        at[0].val.clusterDim.x = C;
+        at[0].val.clusterDim.y = at[0].val.clusterDim.z = 1;
+        cfg.attrs = at;
+        cfg.numAttrs = 1;
+        SA_CUDA(cudaLaunchKernelEx(&cfg, kern, args));
+        count_launch();
+        return SA_OK;
+    });
 }
 
 // block path: one block of 256 threads per instance, two blocks per SM
@@ -979,18 +1009,35 @@ extern "C" sa_status sa_batch_scale(sa_ctx* ctx, int32_t k, const void* const* d
         cnt[b] = (int)m.size();
         order.insert(order.end(), m.begin(), m.end());
     }
-    // K rows buckets: a global slot of K (n x ceil(n/4)*4 floats of the bucket's largest n)
-    // per block, at most two blocks per SM and one per instance
-    std::vector<int> kblocks(plan.count, 0);
-    std::vector<size_t> kslot(plan.count, 0);
+    // the launches: a bucket each, a K rows bucket one per cluster class in it (largest n first);
+    // each of these has a slot per cluster
+    struct Launch {
+        int bucket, first, cnt, cls, clusters;
+        size_t slot;
+    };
+    std::vector<Launch> launches;
     size_t need = align_up((size_t)k * 4, 256) * 3 + align_up((size_t)o->n_p * 8, 256) + 1024 +
-                  SA_BATCH_MAX_BUCKETS * 256;
+                  kBatchLaunches * 256;
     for (int b = 0; b < plan.count; ++b) {
-        if (plan.path[b] != SA_BATCH_KROWS || cnt[b] == 0) continue;
-        const int nmax = hn[members[b].front()];
-        kblocks[b] = std::min(cnt[b], 2 * ctx->num_sms);
-        kslot[b] = (size_t)nmax * align_up((size_t)nmax, 4);
-        need += align_up((size_t)kblocks[b] * kslot[b] * sizeof(float), 256);
+        if (cnt[b] == 0) continue;
+        if (plan.path[b] != SA_BATCH_KROWS) {
+            launches.push_back({b, first[b], cnt[b], -1, 0, 0});
+            continue;
+        }
+        for (int x = 0; x < cnt[b];) {
+            const int cls = cluster_class(hn[members[b][x]]);
+            int y = x;
+            while (y < cnt[b] && cluster_class(hn[members[b][y]]) == cls) ++y;
+            int cap = 0;
+            sa_status crc = cluster_capacity(ctx, cls, wtype, &cap);
+            if (crc) return crc;
+            if (cap < 1) { set_error("batch K rows path: a cluster of %d blocks does not fit", cluster_blocks(cls)); return SA_E_UNSUPPORTED; }
+            const int nmax = hn[members[b][x]];
+            Launch l{b, first[b] + x, y - x, cls, std::min(y - x, cap), 3 * (size_t)nmax * align_up((size_t)nmax, 4)};
+            need += align_up((size_t)l.clusters * l.slot * sizeof(float), 256);
+            launches.push_back(l);
+            x = y;
+        }
     }
     sa_status rc = ctx->ws.reserve(need);
     if (rc) return rc;
@@ -999,41 +1046,38 @@ extern "C" sa_status sa_batch_scale(sa_ctx* ctx, int32_t k, const void* const* d
     int32_t* d_sw = cv.take<int32_t>(k);
     int32_t* d_st = cv.take<int32_t>(k);
     double* d_P = cv.take<double>(o->n_p);
-    unsigned* d_q = cv.take<unsigned>(SA_BATCH_MAX_BUCKETS);
-    std::vector<float*> kscr(plan.count, nullptr);
-    for (int b = 0; b < plan.count; ++b)
-        if (kblocks[b] > 0) kscr[b] = cv.take<float>((size_t)kblocks[b] * kslot[b]);
+    unsigned* d_q = cv.take<unsigned>(kBatchLaunches);
     SA_CUDA(cudaMemcpyAsync(d_order, order.data(), 4 * k, cudaMemcpyHostToDevice, st));
     SA_CUDA(cudaMemcpyAsync(d_P, o->p, 8 * o->n_p, cudaMemcpyHostToDevice, st));
-    SA_CUDA(cudaMemsetAsync(d_q, 0, 4 * SA_BATCH_MAX_BUCKETS, st));
-    // fork: each non-empty bucket launches on a stream of its own after the set-up above,
-    // so the buckets' kernels run side by side; the context stream waits for all of them
-    if (!ctx->batch_events[SA_BATCH_MAX_BUCKETS])
-        SA_CUDA(cudaEventCreateWithFlags(&ctx->batch_events[SA_BATCH_MAX_BUCKETS], cudaEventDisableTiming));
-    SA_CUDA(cudaEventRecord(ctx->batch_events[SA_BATCH_MAX_BUCKETS], st));
-    for (int b = 0; b < plan.count; ++b) {
-        if (cnt[b] == 0) continue;
-        if (!ctx->batch_streams[b]) SA_CUDA(cudaStreamCreateWithFlags(&ctx->batch_streams[b], cudaStreamNonBlocking));
-        if (!ctx->batch_events[b]) SA_CUDA(cudaEventCreateWithFlags(&ctx->batch_events[b], cudaEventDisableTiming));
-        cudaStream_t bs = ctx->batch_streams[b];
-        SA_CUDA(cudaStreamWaitEvent(bs, ctx->batch_events[SA_BATCH_MAX_BUCKETS], 0));
+    SA_CUDA(cudaMemsetAsync(d_q, 0, 4 * kBatchLaunches, st));
+    // fork: each launch goes to a stream of its own after the set-up above, so that they run
+    // side by side; the context stream waits for all of them
+    if (!ctx->batch_events[kBatchLaunches])
+        SA_CUDA(cudaEventCreateWithFlags(&ctx->batch_events[kBatchLaunches], cudaEventDisableTiming));
+    SA_CUDA(cudaEventRecord(ctx->batch_events[kBatchLaunches], st));
+    for (int x = 0; x < (int)launches.size(); ++x) {
+        const Launch& l = launches[x];
+        const int b = l.bucket;
+        if (!ctx->batch_streams[x]) SA_CUDA(cudaStreamCreateWithFlags(&ctx->batch_streams[x], cudaStreamNonBlocking));
+        if (!ctx->batch_events[x]) SA_CUDA(cudaEventCreateWithFlags(&ctx->batch_events[x], cudaEventDisableTiming));
+        cudaStream_t bs = ctx->batch_streams[x];
+        SA_CUDA(cudaStreamWaitEvent(bs, ctx->batch_events[kBatchLaunches], 0));
         const auto& m = members[b];
-        const bool desc = plan.path[b] == SA_BATCH_BLOCK || plan.path[b] == SA_BATCH_KROWS;
-        const int nmax = desc ? hn[m.front()] : hn[m.back()];
-        BatchArgs args{d_w, d_n, d_ld, d_off, d_order + first[b], cnt[b], wtype == SA_I16, d_P, o->n_p, o->tol,
-                       o->max_sweeps_per_p, d_u, d_v, d_sw, d_st, d_q + b, 0, nullptr, 0};
+        const int nmax = plan.path[b] == SA_BATCH_BLOCK ? hn[m.front()] : hn[m.back()];
+        BatchArgs args{d_w, d_n, d_ld, d_off, d_order + l.first, l.cnt, wtype == SA_I16, d_P, o->n_p, o->tol,
+                       o->max_sweeps_per_p, d_u, d_v, d_sw, d_st, d_q + x, 0, nullptr, 0};
         if (plan.path[b] == SA_BATCH_GROUP)
             rc = launch_group_path(ctx, bs, args, nmax, plan.warps[b], plan.per_block[b], wtype);
         else if (plan.path[b] == SA_BATCH_REGS)
             rc = launch_regs_path(ctx, bs, args, nmax, plan.warps[b], plan.per_block[b], wtype);
         else if (plan.path[b] == SA_BATCH_KROWS) {
-            args.kscr = kscr[b];
-            args.kscr_floats = kslot[b];
-            rc = launch_krows_path(ctx, bs, args, nmax, kblocks[b], wtype);
+            args.kscr = cv.take<float>((size_t)l.clusters * l.slot);
+            args.kscr_floats = l.slot;
+            rc = launch_cluster_path(bs, args, l.cls, l.clusters, wtype);
         } else rc = launch_block_path(ctx, bs, args, nmax, wtype);
         // joined even after a failed launch: the buckets already running finish first
-        SA_CUDA(cudaEventRecord(ctx->batch_events[b], bs));
-        SA_CUDA(cudaStreamWaitEvent(st, ctx->batch_events[b], 0));
+        SA_CUDA(cudaEventRecord(ctx->batch_events[x], bs));
+        SA_CUDA(cudaStreamWaitEvent(st, ctx->batch_events[x], 0));
         if (rc) {
             cudaStreamSynchronize(st);
             return rc;

@@ -1,7 +1,8 @@
 // krows.cuh -- one instance of the batched form on one block of 256 threads, on the
 // per-step matrix K (Sec. 4.1.2 iteration in log coordinates, Sec. 4.2 stop rule, the
-// deformed warm start of Sec. 4.1 between p steps).  Used by the batched launch
-// (sa_batch_scale's K rows path) and by the server's device-resident request queue.
+// deformed warm start of Sec. 4.1 between p steps).  Used by the server's device-resident
+// request queue, whose blocks take one request each (the batched launch spreads an instance
+// over a cluster instead, batch_cluster.cuh).
 //
 // K rows path: the larger instances (n <= 128 CH) one per block of 256 threads, on the
 // per-step matrix K of the step path in a global-memory slot of the block (n x ceil(n/4)*4

@@ -71,6 +71,10 @@ struct PinnedBuf {
     ~PinnedBuf();
 };
 
+// launches of one sa_batch_scale at most: one per bucket and, since a K rows bucket is split where
+// the blocks of an instance change, three more
+constexpr int kBatchLaunches = SA_BATCH_MAX_BUCKETS + 3;
+
 // sa_batch_scale's plan when none is set (see sa_set_batch_plan)
 inline sa_batch_plan default_batch_plan() {
     sa_batch_plan p{};
@@ -104,8 +108,8 @@ struct sa_ctx {
                                               // policy (the rest "evict first")
     int test_unreachable_barrier = 0;         // testing hook (SA_OPT_TEST_UNREACHABLE_BARRIER)
     sa_batch_plan batch_plan = sa::default_batch_plan();
-    cudaStream_t batch_streams[SA_BATCH_MAX_BUCKETS] = {};   // one per bucket launch (lazily made)
-    cudaEvent_t batch_events[SA_BATCH_MAX_BUCKETS + 1] = {};
+    cudaStream_t batch_streams[sa::kBatchLaunches] = {};   // one per launch (lazily made)
+    cudaEvent_t batch_events[sa::kBatchLaunches + 1] = {};
     sa::Workspace ws;        // scratch for sweeps, prune, certify
     sa::Workspace input;     // device copy of host inputs (sa_assign_host)
     sa::Workspace keep;      // sa_scale: the caller's warm-start potentials, restored on failure

@@ -259,3 +259,57 @@ def test_plans_are_checked_and_applied(ctx):
 def test_batch_rejects_large_n(ctx):
     rc, *_ = batch_scale(ctx, [W.uniform(600, 1, 1000, 3, dtype=np.int16)], [1.0])
     assert rc == L.SA_E_UNSUPPORTED
+
+
+KROWS_SIZES = [1, 3, 31, 130, 143, 144, 145, 200, 255, 256, 257, 321, 383, 384, 385, 450, 509, 512]
+
+
+@pytest.mark.parametrize("dtype", [np.int16, np.int32])
+def test_krows_cluster_shapes(ctx, dtype):
+    """The K rows path at the edges of its shapes (one block up to 144, clusters of two up to 256
+    and 384, of four up to 512), several instances a cluster, absent entries, columns of very
+    different mass and one weight above the log2 table: the path's tolerances."""
+    mats = []
+    for q, n in enumerate(KROWS_SIZES * 2):
+        m = W.uniform(n, 1, 1000 if dtype == np.int16 else 1 << 20, 1700 + q, dtype=dtype)
+        if n > 16:
+            m[::3, 1::7] = 0
+            m[:, n // 2:] = np.maximum(m[:, n // 2:] >> 4, (m[:, n // 2:] > 0).astype(dtype))
+        mats.append(m)
+    ps = [1.0, 2.0, 4.0, 8.0]
+    rc, us, vs, sw, st = batch_scale(ctx, mats, ps, plan=[(512, "krows", 0, 0)])
+    assert rc == 0 and np.all(st == 0), (rc, st)
+    for m, u, v in zip(mats, us, vs):
+        b = oracle.log_weights(m.astype(np.int64))
+        uo, vo, swo, rso, sto = oracle.sinkhorn(b, ps, 1e-6, 20000)
+        r, c = oracle.sums(b, ps[-1], u, v)
+        assert max(np.abs(r - 1).max(), np.abs(c - 1).max()) < 2e-6, m.shape
+        xo = oracle.xmatrix(b, ps[-1], uo, vo)
+        xg = oracle.xmatrix(b, ps[-1], u, v)
+        assert np.all(np.abs(xg - xo) <= 8e-6 * np.maximum(xo, 1.0 / m.shape[0]) + 1e-9), m.shape
+
+
+def test_krows_clusters_report_empty_rows_and_columns(ctx):
+    """An empty row or column ends its instance with status -6 in every shape, in whichever
+    block of the cluster it lies, and leaves its neighbours alone."""
+    mats, want = [], []
+    for n in (100, 200, 300, 500):
+        for kind in ("none", "first row", "last row", "first column", "last column"):
+            m = W.uniform(n, 1, 1000, 1800 + n, dtype=np.int16)
+            if kind == "first row":
+                m[0, :] = 0
+            elif kind == "last row":
+                m[-1, :] = 0
+            elif kind == "first column":
+                m[:, 0] = 0
+            elif kind == "last column":
+                m[:, -1] = 0
+            mats.append(m)
+            want.append(0 if kind == "none" else -6)
+    rc, us, vs, sw, st = batch_scale(ctx, mats, [1.0, 2.0], plan=[(512, "krows", 0, 0)])
+    assert rc == L.SA_E_NONFINITE
+    assert list(st) == want
+    for m, u, v, s in zip(mats, us, vs, want):
+        if s == 0:
+            r, c = oracle.sums(oracle.log_weights(m.astype(np.int64)), 2.0, u, v)
+            assert max(np.abs(r - 1).max(), np.abs(c - 1).max()) < 2e-6
