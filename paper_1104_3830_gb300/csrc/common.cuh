@@ -1,7 +1,7 @@
 // common.cuh -- device helpers shared by the libsa kernels (sm_103a).
 //
 // SFU wrappers, integer-weight decoding, warp reductions, shared-memory barriers for the
-// bulk-copy engine, and a bounded group barrier for persistent cooperative kernels.
+// bulk-copy engine, and a bounded grid barrier for persistent cooperative kernels.
 // Every spin-wait here is bounded by a wall-clock limit; on expiry it records an error
 // code and returns false so the kernel can drain and exit.
 #pragma once
@@ -81,42 +81,28 @@ __device__ __forceinline__ void st_release(unsigned* p, unsigned v) {
     asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
 }
 
-// Barrier over `nblocks` co-resident blocks (cooperative launch).  bar[0] counts
-// arrivals, bar[1] is the generation.  Returns false if the wait exceeded timeout_ns
-// or another block already reported an error; *err then holds a kErr* code.
-__device__ __forceinline__ bool group_barrier(unsigned* bar, unsigned nblocks, int* err,
-                                              uint64_t timeout_ns) {
-    __shared__ int s_ok;
+// Barrier over the co-resident blocks of a cooperative launch on a counter that only grows
+// (target: arrivals once every block has come).  Thread 0 arrives with a release reduction,
+// which carries the block's writes ordered before it by the block barrier, and polls with
+// acquire loads: no returning atomic, no fence, no second word.  Returns false if the wait
+// exceeded wait_ns or another block reported an error.
+__device__ __forceinline__ bool counter_sync(unsigned* ctr, unsigned target, int* err, int* s_ok, uint64_t wait_ns) {
     __syncthreads();
     if (threadIdx.x == 0) {
         int ok = 1;
-        unsigned gen = ld_acquire(bar + 1);
-        __threadfence();
-        unsigned prev = atomicAdd(bar, 1u);
-        if (prev == nblocks - 1) {
-            atomicExch(bar, 0u);
-            __threadfence();
-            st_release(bar + 1, gen + 1);
-        } else {
-            uint64_t t0 = globaltimer_ns();
-            unsigned spins = 0;
-            while (ld_acquire(bar + 1) == gen) {
-                if ((++spins & 63u) == 0) {
-                    if (*(volatile int*)err != 0) { ok = 0; break; }
-                    if (globaltimer_ns() - t0 > timeout_ns) {
-                        atomicCAS(err, 0, kErrTimeout);
-                        ok = 0;
-                        break;
-                    }
-                }
-                __nanosleep(20);
+        asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(ctr), "r"(1u) : "memory");
+        const uint64_t t0 = globaltimer_ns();
+        unsigned spins = 0;
+        while (ld_acquire(ctr) < target) {
+            if ((++spins & 31u) == 0) {
+                if (*(volatile int*)err != 0) { ok = 0; break; }
+                if (globaltimer_ns() - t0 > wait_ns) { atomicCAS(err, 0, kErrTimeout); ok = 0; break; }
             }
         }
-        if (*(volatile int*)err != 0) ok = 0;
-        s_ok = ok;
+        *s_ok = ok;
     }
     __syncthreads();
-    return s_ok != 0;
+    return *s_ok != 0;
 }
 
 // ---- shared-memory barriers and the bulk-copy (TMA) engine ----------------------------

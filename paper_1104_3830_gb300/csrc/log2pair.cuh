@@ -24,6 +24,13 @@ __device__ __forceinline__ float two_sum(float a, float b, float* err) {
     return s;
 }
 
+// the sum of two unevaluated pairs (to about 2^-47)
+__device__ __forceinline__ void pair_add(float& hi, float& lo, float h2, float l2) {
+    float e;
+    hi = two_sum(hi, h2, &e);
+    lo = (lo + l2) + e;
+}
+
 // Shared table for log2 of a weight: entry j (the top 8 mantissa bits of m in [1, 2)) holds
 // g_j = 1 / (1 + (j + 0.5)/256) rounded to 9 significant bits and -log2(g_j) as a float pair.
 __device__ __forceinline__ float4 log2_tab_entry(int j) {

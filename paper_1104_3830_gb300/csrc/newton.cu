@@ -68,6 +68,7 @@ struct NtState {
     int newton_it;
     int stall;       // Newton steps since the residual last fell below half of res_ref
     double tau, res, gamma, gamma0, gamma_prev, alpha, alpha_prev, beta, thr;
+    double corr;     // beta gamma / alpha_prev of the next CG step
     double res_ref;
 };
 
@@ -103,9 +104,9 @@ struct NtArgs {
     float* rf;
     double* prt;    // T x n row partials
     float* pc;      // R x ldk column partials
-    double* bred;   // finalisation block partials (4 per block)
-    double* cred;   // update block partials (4 per block)
-    unsigned* bar;  // grid barrier (count, generation)
+    float* bred;    // finalisation block partials (8 per block: two pairs and a minimum)
+    float* cred;    // update block partials
+    unsigned* bar;  // grid barrier counter
     int* err;       // kErr* code of a failed wait or step
 };
 
@@ -242,7 +243,7 @@ __global__ void __launch_bounds__(kNtThreads) nt_kwrite_kernel(const WT* __restr
 // over the 8 warps of the block; each lane issues its loads in batches of 24 independent
 // loads.
 template <bool MAX>
-__device__ __forceinline__ double nt_stripes(const float* __restrict__ pc, int R, int ldk, int j, int wid) {
+__device__ __forceinline__ float2 nt_stripes(const float* __restrict__ pc, int R, int ldk, int j, int wid) {
     constexpr int kB = 24;
     float acc = 0.0f, comp = 0.0f;   // 0 is also the identity of the max: the partials are >= 0
     for (int base = wid; base < R; base += kNtWarps * kB) {
@@ -264,7 +265,7 @@ __device__ __forceinline__ double nt_stripes(const float* __restrict__ pc, int R
             }
         }
     }
-    return MAX ? (double)acc : (double)acc - (double)comp;   // the compensated sum in FP64
+    return make_float2(acc, MAX ? 0.0f : -comp);   // the compensated sum as a pair
 }
 
 // starting point of a p step: rho = 1, kappa_j = 1 / max_i K_ij.
@@ -275,7 +276,7 @@ __global__ void __launch_bounds__(kNtThreads) nt_init_kernel(NtArgs A) {
     const int nbc = (n + 31) / 32;
     if ((int)blockIdx.x < nbc) {
         const int j = blockIdx.x * 32 + lane;
-        sred[wid][lane] = j < n ? (float)nt_stripes<true>(A.pc, A.R, A.ldk, j, wid) : 0.0f;
+        sred[wid][lane] = j < n ? nt_stripes<true>(A.pc, A.R, A.ldk, j, wid).x : 0.0f;
         __syncthreads();
         if (wid == 0 && j < n) {
             float m = 0.0f;
@@ -297,11 +298,15 @@ __global__ void __launch_bounds__(kNtThreads) nt_init_kernel(NtArgs A) {
     }
 }
 
+// The reductions below add FP32 values as unevaluated FP32 pairs (to about 2^-47) and turn to FP64
+// once, at their end: a chain of FP64 additions costs about a hundred cycles a link on GB300,
+// and the phases between two applications of the operator were mostly such chains (rows, stripes,
+// block and grid reductions: 16 thousand cycles of an iteration at n = 3001).
+
 // Block reduction of three FP32 values at once: v0 by max (MAX0) or sum, v1 by sum, v2 by
-// min; the warp results are combined in FP64 by thread 0, where the results are valid.
+// min; thread 0 writes the block's partial (pairs of v0 and v1, then v2).
 template <bool MAX0>
-__device__ __forceinline__ void nt_block_reduce3(float v0, float v1, float v2, float (*sh)[kNtWarps],
-                                                 double* o0, double* o1, double* o2) {
+__device__ __forceinline__ void nt_block_reduce3(float v0, float v1, float v2, float (*sh)[kNtWarps], float* out) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
         const float u0 = __shfl_xor_sync(0xffffffffu, v0, o);
@@ -309,47 +314,55 @@ __device__ __forceinline__ void nt_block_reduce3(float v0, float v1, float v2, f
         v1 += __shfl_xor_sync(0xffffffffu, v1, o);
         v2 = fminf(v2, __shfl_xor_sync(0xffffffffu, v2, o));
     }
-    __syncthreads();   // sh may still be read by thread 0 of the previous reduction
-    if ((threadIdx.x & 31) == 0) {
+    __syncthreads();   // sh may still be read by warp 0 of the previous reduction
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) {
         sh[0][threadIdx.x >> 5] = v0;
         sh[1][threadIdx.x >> 5] = v1;
         sh[2][threadIdx.x >> 5] = v2;
     }
     __syncthreads();
-    if (threadIdx.x == 0) {
-        double r0 = sh[0][0], r1 = sh[1][0], r2 = sh[2][0];
-        for (int k = 1; k < kNtWarps; ++k) {
-            r0 = MAX0 ? fmax(r0, (double)sh[0][k]) : r0 + sh[0][k];
-            r1 += sh[1][k];
-            r2 = fmin(r2, (double)sh[2][k]);
+    if (threadIdx.x < 32) {
+        const int x = lane & (kNtWarps - 1);
+        float h0 = sh[0][x], l0 = 0.0f, h1 = sh[1][x], l1 = 0.0f, m = sh[2][x];
+#pragma unroll
+        for (int o = 1; o < kNtWarps; o <<= 1) {
+            const float u0 = __shfl_xor_sync(0xffffffffu, h0, o), w0 = __shfl_xor_sync(0xffffffffu, l0, o);
+            if (MAX0) h0 = fmaxf(h0, u0);
+            else pair_add(h0, l0, u0, w0);
+            pair_add(h1, l1, __shfl_xor_sync(0xffffffffu, h1, o), __shfl_xor_sync(0xffffffffu, l1, o));
+            m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
         }
-        *o0 = r0;
-        *o1 = r1;
-        *o2 = r2;
+        if (lane == 0) {
+            *(float4*)out = make_float4(h0, l0, h1, l1);
+            out[4] = m;
+        }
     }
 }
 
-// Reduction of the G block partials (4 doubles each, the first three used) by warp 0 in a
-// fixed order, so that every block obtains identical values; valid in lane 0 of warp 0.
+// Reduction of the G block partials by warp 0 in a fixed order, so that every block obtains
+// identical values; valid in lane 0 of warp 0.
 template <bool MAX0>
-__device__ __forceinline__ void nt_grid_reduce3(const double* part, int G, double* g0, double* g1, double* g2) {
-    double a0 = 0.0, a1 = 0.0, a2 = INFINITY;   // 0 is also the identity of the max of |v - 1|
+__device__ __forceinline__ void nt_grid_reduce3(const float* part, int G, double* g0, double* g1, double* g2) {
+    float h0 = 0.0f, l0 = 0.0f, h1 = 0.0f, l1 = 0.0f, m = INFINITY;   // 0 is also the identity of the max of |v - 1|
     for (int x = threadIdx.x; x < G; x += 32) {
-        const double x0 = __ldcg(part + 4 * x);
-        a0 = MAX0 ? fmax(a0, x0) : a0 + x0;
-        a1 += __ldcg(part + 4 * x + 1);
-        a2 = fmin(a2, __ldcg(part + 4 * x + 2));
+        const float4 q = __ldcg((const float4*)(part + 8 * x));
+        if (MAX0) h0 = fmaxf(h0, q.x);
+        else pair_add(h0, l0, q.x, q.y);
+        pair_add(h1, l1, q.z, q.w);
+        m = fminf(m, __ldcg(part + 8 * x + 4));
     }
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) {
-        const double u0 = __shfl_xor_sync(0xffffffffu, a0, o);
-        a0 = MAX0 ? fmax(a0, u0) : a0 + u0;
-        a1 += __shfl_xor_sync(0xffffffffu, a1, o);
-        a2 = fmin(a2, __shfl_xor_sync(0xffffffffu, a2, o));
+        const float u0 = __shfl_xor_sync(0xffffffffu, h0, o), w0 = __shfl_xor_sync(0xffffffffu, l0, o);
+        if (MAX0) h0 = fmaxf(h0, u0);
+        else pair_add(h0, l0, u0, w0);
+        pair_add(h1, l1, __shfl_xor_sync(0xffffffffu, h1, o), __shfl_xor_sync(0xffffffffu, l1, o));
+        m = fminf(m, __shfl_xor_sync(0xffffffffu, m, o));
     }
-    *g0 = a0;
-    *g1 = a1;
-    *g2 = a2;
+    *g0 = MAX0 ? (double)h0 : (double)h0 + (double)l0;
+    *g1 = (double)h1 + (double)l1;
+    *g2 = (double)m;
 }
 
 // Decisions after the finalisation (g0: max |v - 1| or sum w r; g1: sum (1 - v)^2;
@@ -392,13 +405,7 @@ __device__ __forceinline__ void nt_after_fin(NtState& S, bool res_mode, double g
         }
     } else {
         // Chronopoulos-Gear: alpha = gamma / (delta - beta gamma / alpha_prev), delta = r.Mr
-        if (S.first) {
-            S.beta = 0.0;
-            S.alpha = S.gamma / g0;
-        } else {
-            S.beta = S.gamma / S.gamma_prev;
-            S.alpha = S.gamma / (g0 - S.beta * S.gamma / S.alpha_prev);
-        }
+        S.alpha = S.gamma / (g0 - S.corr);   // corr = beta gamma / alpha_prev, 0 in the first step
         if (!(S.alpha > 0.0 && S.alpha < INFINITY)) {
             S.alpha = 0.0;
             S.breakdown = 1;
@@ -441,8 +448,9 @@ __host__ __device__ inline size_t nt_smem_bytes(int ch, int rows_per, int own) {
 template <int CH>
 __global__ void __launch_bounds__(kNtThreads, 2) nt_solve_kernel(NtArgs A, double tol, int cap,
                                                                  NtOut* out) {
-    __shared__ double sred[kNtWarps][33];
+    __shared__ float2 sred[kNtWarps][33];
     __shared__ float sh[3][kNtWarps];
+    __shared__ int s_ok;
     __shared__ NtState S;
     __shared__ __align__(8) uint64_t full[kNtStages];   // a slot's row tile has landed
     __shared__ unsigned rel_cnt[kNtStages];               // warp releases of a slot
@@ -511,6 +519,7 @@ __global__ void __launch_bounds__(kNtThreads, 2) nt_solve_kernel(NtArgs A, doubl
     if (tid == 0)
         for (uint32_t v = 0; v < (uint32_t)kNtStages; ++v) issue(v);
     uint32_t vbase = 0;   // ring index of the phase's first row
+    unsigned nbar = 0;    // grid barriers passed
     for (;;) {
         const bool res_mode = S.mode == kNtRes;
         const bool apply = S.apply != 0;
@@ -573,10 +582,10 @@ __global__ void __launch_bounds__(kNtThreads, 2) nt_solve_kernel(NtArgs A, doubl
             vbase += (uint32_t)nrows;
             __syncthreads();
             for (int i = tid; i < nrows; i += kNtThreads) {
-                double sm = 0.0;
+                float hi = 0.0f, lo = 0.0f;
 #pragma unroll
-                for (int x = 0; x < kNtWarps; ++x) sm += (double)rowdot[i * kNtWarps + x];
-                A.prt[(int64_t)t * n + r0 + i] = sm;
+                for (int x = 0; x < kNtWarps; ++x) pair_add(hi, lo, rowdot[i * kNtWarps + x], 0.0f);
+                A.prt[(int64_t)t * n + r0 + i] = (double)hi + (double)lo;
             }
 #pragma unroll
             for (int k = 0; k < CH; ++k)
@@ -584,18 +593,22 @@ __global__ void __launch_bounds__(kNtThreads, 2) nt_solve_kernel(NtArgs A, doubl
                     *(float4*)(A.pc + (int64_t)s * A.ldk + 4 * q[k]) =
                         make_float4(acc[4 * k], acc[4 * k + 1], acc[4 * k + 2], acc[4 * k + 3]);
         }
-        if (s_fail) atomicCAS(A.err, 0, kErrTimeout);   // a ring wait gave up: every block stops
-        if (!group_barrier(A.bar, G, A.err, kWaitTimeoutNs)) break;
+        if (s_fail) {   // a ring wait gave up: the others find the error while they wait for this block
+            atomicCAS(A.err, 0, kErrTimeout);
+            break;
+        }
+        if (!counter_sync(A.bar, ++nbar * (unsigned)G, A.err, &s_ok, kWaitTimeoutNs)) break;
         // ---- B: finalise the owned entries: m = D(x) S D(x) z; v, r, y or w ----
         {
             for (int cb = c0; cb < c1; cb += 32) {
                 const int j = cb + lane;
-                sred[wid][lane] = j < c1 ? nt_stripes<false>(A.pc, A.R, A.ldk, j, wid) : 0.0;
+                sred[wid][lane] = j < c1 ? nt_stripes<false>(A.pc, A.R, A.ldk, j, wid) : make_float2(0.0f, 0.0f);
                 __syncthreads();
                 if (wid == 0 && j < c1) {
-                    double tot = 0.0;
-                    for (int x = 0; x < kNtWarps; ++x) tot += sred[x][lane];
-                    tot_s[j - c0] = tot;
+                    float hi = 0.0f, lo = 0.0f;
+#pragma unroll
+                    for (int x = 0; x < kNtWarps; ++x) pair_add(hi, lo, sred[x][lane].x, sred[x][lane].y);
+                    tot_s[j - c0] = (double)hi + (double)lo;
                 }
                 __syncthreads();
             }
@@ -637,22 +650,25 @@ __global__ void __launch_bounds__(kNtThreads, 2) nt_solve_kernel(NtArgs A, doubl
                     a2 = fminf(a2, (we > -INFINITY && we < INFINITY) ? 1.0f : -1.0f);
                 }
             }
-            double b0, b1, b2;
-            if (res_mode) nt_block_reduce3<true>(a0, a1, a2, sh, &b0, &b1, &b2);
-            else nt_block_reduce3<false>(a0, a1, a2, sh, &b0, &b1, &b2);
-            if (tid == 0) {
-                A.bred[4 * b] = b0;
-                A.bred[4 * b + 1] = b1;
-                A.bred[4 * b + 2] = b2;
-            }
+            if (res_mode) nt_block_reduce3<true>(a0, a1, a2, sh, A.bred + 8 * b);
+            else nt_block_reduce3<false>(a0, a1, a2, sh, A.bred + 8 * b);
         }
-        if (!group_barrier(A.bar, G, A.err, kWaitTimeoutNs)) break;
+        if (!counter_sync(A.bar, ++nbar * (unsigned)G, A.err, &s_ok, kWaitTimeoutNs)) break;
         // ---- C: every block reduces all partials in the same order: same decisions ----
+        // (the divisions that do not need g0 on another warp meanwhile)
         if (wid == 0) {
             double g0, g1, g2;
             if (res_mode) nt_grid_reduce3<true>(A.bred, G, &g0, &g1, &g2);
             else nt_grid_reduce3<false>(A.bred, G, &g0, &g1, &g2);
+            asm volatile("bar.sync 1, 64;" ::: "memory");
             if (lane == 0) nt_after_fin(S, res_mode, g0, g1, g2, tol, cap);
+        } else if (wid == 1) {
+            if (lane == 0 && !res_mode) {
+                const double beta = S.first ? 0.0 : S.gamma / S.gamma_prev;
+                S.beta = beta;
+                S.corr = S.first ? 0.0 : beta * S.gamma / S.alpha_prev;
+            }
+            asm volatile("bar.sync 1, 64;" ::: "memory");
         }
         __syncthreads();
         if (S.mode == kNtDone) break;
@@ -678,15 +694,9 @@ __global__ void __launch_bounds__(kNtThreads, 2) nt_solve_kernel(NtArgs A, doubl
                 rr += (float)(rn * rn);
                 ymin = fminf(ymin, (float)ye);
             }
-            double b0, b1, b2;
-            nt_block_reduce3<false>(rr, 0.0f, ymin, sh, &b0, &b1, &b2);
-            if (tid == 0) {
-                A.cred[4 * b] = b0;
-                A.cred[4 * b + 1] = 0.0;
-                A.cred[4 * b + 2] = b2;
-            }
+            nt_block_reduce3<false>(rr, 0.0f, ymin, sh, A.cred + 8 * b);
         }
-        if (!group_barrier(A.bar, G, A.err, kWaitTimeoutNs)) break;
+        if (!counter_sync(A.bar, ++nbar * (unsigned)G, A.err, &s_ok, kWaitTimeoutNs)) break;
         if (wid == 0) {
             double g0, g1, g2;
             nt_grid_reduce3<false>(A.cred, G, &g0, &g1, &g2);
@@ -822,8 +832,8 @@ sa_status scale_newton(sa_ctx* ctx, const sa_matrix* a, const sa_scale_opts* o, 
     A.rf = cv.take<float>(2 * (size_t)n);
     A.prt = cv.take<double>((size_t)P.T * n);
     A.pc = cv.take<float>((size_t)P.R * ldk);
-    A.bred = cv.take<double>((size_t)P.grid * 4);
-    A.cred = cv.take<double>((size_t)P.grid * 4);
+    A.bred = cv.take<float>((size_t)P.grid * 8);
+    A.cred = cv.take<float>((size_t)P.grid * 8);
     NtOut* d_out = cv.take<NtOut>(o->n_p);
     float4* tab = cv.take<float4>(256);
     float2* vp = cv.take<float2>(n);

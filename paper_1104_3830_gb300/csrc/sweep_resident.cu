@@ -117,26 +117,6 @@ struct PollLimit {
     }
 };
 
-// Grid barrier between p steps (see step_grid_sync in sweep_step.cu).
-__device__ __forceinline__ bool res_grid_sync(unsigned* ctr, unsigned target, int* err, int* s_ok, uint64_t wait_ns) {
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        int ok = 1;
-        asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(ctr), "r"(1u) : "memory");
-        const uint64_t t0 = globaltimer_ns();
-        unsigned spins = 0;
-        while (ld_acquire(ctr) < target) {
-            if ((++spins & 31u) == 0) {
-                if (*(volatile int*)err != 0) { ok = 0; break; }
-                if (globaltimer_ns() - t0 > wait_ns) { atomicCAS(err, 0, kErrTimeout); ok = 0; break; }
-            }
-        }
-        *s_ok = ok;
-    }
-    __syncthreads();
-    return *s_ok != 0;
-}
-
 __device__ __forceinline__ unsigned float_key(float x) {
     const unsigned b = __float_as_uint(x);
     return (b & 0x80000000u) ? ~b : (b | 0x80000000u);
@@ -167,13 +147,6 @@ __device__ __forceinline__ void res_load4(const ResArgs& A, int row, int j, int 
             for (int e = 0; e < 4; ++e) w[e] = e < cnt ? p[e] : 0;
         }
     }
-}
-
-// the sum of two unevaluated pairs
-__device__ __forceinline__ void pair_add(float& hi, float& lo, float h2, float l2) {
-    float e;
-    hi = two_sum(hi, h2, &e);
-    lo = (lo + l2) + e;
 }
 
 // log2 of s = hi + lo > 0 as a pair, to about 2^-46: the reduction of sum_log2 in FP32 (m g - 1
@@ -277,7 +250,7 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
         s_dec[0] = s_dec[1] = 0u;
     }
     unsigned nbar = 1;
-    if (!res_grid_sync(A.bar, nbar * (unsigned)G + A.extra_arrivals, A.err, &s_ok, A.wait_ns)) return;
+    if (!counter_sync(A.bar, nbar * (unsigned)G + A.extra_arrivals, A.err, &s_ok, A.wait_ns)) return;
 
     if (wid == NW) {
         // ---- the potentials' warp: lane l owns column c0 + l ----
@@ -321,7 +294,7 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
             }
             if (!last) {
                 ++nbar;
-                if (!res_grid_sync(A.bar, nbar * (unsigned)G + A.extra_arrivals, A.err, &s_ok, A.wait_ns)) return;
+                if (!counter_sync(A.bar, nbar * (unsigned)G + A.extra_arrivals, A.err, &s_ok, A.wait_ns)) return;
             }
         }
         return;
@@ -725,7 +698,7 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
         if (b == 0 && tid == 0) A.sweeps_out[k] = sweeps;
         if (!last) {
             ++nbar;
-            if (!res_grid_sync(A.bar, nbar * (unsigned)G + A.extra_arrivals, A.err, &s_ok, A.wait_ns)) return;
+            if (!counter_sync(A.bar, nbar * (unsigned)G + A.extra_arrivals, A.err, &s_ok, A.wait_ns)) return;
         }
     }
 }
