@@ -63,13 +63,42 @@ __device__ __forceinline__ float2 log2_pair(int w, const float4* tab) {
     return make_float2(s2, ((e1 + e2) + t.z) + small);
 }
 
-// log2 of a positive integer weight as a float pair (shared table + series for the int16
-// range; FP64 above it)
+// log2 of s = hi + lo > 0 as a pair, to about 2^-46 (rms; 2^-43.7 at most): the reduction of sum_log2 in FP32 (m g - 1
+// is exact: 24 + 8 bits of which the leading 8 cancel)
+__device__ __forceinline__ float2 pair_log2(float hi, float lo, const float4* tab) {
+    const unsigned bits = __float_as_uint(hi);
+    const int e = (int)(bits >> 23) - 127;
+    const float d = hi - 1.0f;
+    const bool near = fabsf(d) < 0x1p-8f;
+    const float4 t = tab[(bits >> 15) & 0xffu];
+    const float m = __uint_as_float((bits & 0x7fffffu) | 0x3f800000u);
+    const float scale = __uint_as_float((unsigned)(min(max(-e, -126), 126) + 127) << 23);
+    const float r = near ? d : fmaf(m, t.x, -1.0f);
+    const float rl = near ? lo : lo * scale * t.x;
+    const float b0 = near ? 0.0f : (float)e, b1 = near ? 0.0f : t.y, b2 = near ? 0.0f : t.z;
+    const float l2eh = 1.4426950216293335f, l2el = 1.925963033500011e-08f;   // log2(e) as a pair
+    // ln(1 + r + rl) = a + tail, the square split exactly, the cubic and the rest below 2^-23
+    const float q = r * r, qe = fmaf(r, r, -q);
+    float e0, e1, e2;
+    const float a = two_sum(r, -0.5f * q, &e0);
+    const float cub = q * r * (0.333333343f + r * (-0.25f + r * (0.2f + r * -0.166666672f)));
+    const float tail = (e0 - 0.5f * qe) + (fmaf(rl, q - r, rl) + cub);
+    const float ph = a * l2eh;
+    const float pe = fmaf(tail, l2eh, fmaf(a, l2el, fmaf(a, l2eh, -ph)));
+    const float s1 = two_sum(b1, ph, &e1);   // both below 1: the exponent's addition rounds last
+    const float s2 = two_sum(b0, s1, &e2);
+    return make_float2(s2, ((e1 + b2) + pe) + e2);
+}
+
+// log2 of a positive integer weight as a float pair, from the shared table: the short series for
+// the int16 range, the longer one above it, where a weight is a float and an exact remainder.  (An
+// FP64 logarithm there took the first evaluation of K about 45 FP64 instructions an entry, at two
+// of them per clock and SM: 0.4 ms of 2.8 at n = 2047, and growing as n^2.)  Both carry log2 w at
+// least as closely as the pair's own second part does above the int16 range (2^-44).
 __device__ __forceinline__ float2 wlog2(const float4* stab, int w) {
     if (w < kLog2Tab) return log2_pair(w, stab);
-    const double l = log2((double)w);
-    const float hi = (float)l;
-    return make_float2(hi, (float)(l - (double)hi));
+    const float hi = (float)w;                                   // up to 2^31
+    return pair_log2(hi, (float)(int)((unsigned)w - (unsigned)hi), stab);
 }
 
 // 2^(p log2 w - V_j - m) with the operands as float pairs (p = ph + pl): the large leading

@@ -149,33 +149,6 @@ __device__ __forceinline__ void res_load4(const ResArgs& A, int row, int j, int 
     }
 }
 
-// log2 of s = hi + lo > 0 as a pair, to about 2^-46: the reduction of sum_log2 in FP32 (m g - 1
-// is exact: 24 + 8 bits of which the leading 8 cancel)
-__device__ __forceinline__ float2 pair_log2(float hi, float lo, const float4* tab) {
-    const unsigned bits = __float_as_uint(hi);
-    const int e = (int)(bits >> 23) - 127;
-    const float d = hi - 1.0f;
-    const bool near = fabsf(d) < 0x1p-8f;
-    const float4 t = tab[(bits >> 15) & 0xffu];
-    const float m = __uint_as_float((bits & 0x7fffffu) | 0x3f800000u);
-    const float scale = __uint_as_float((unsigned)(min(max(-e, -126), 126) + 127) << 23);
-    const float r = near ? d : fmaf(m, t.x, -1.0f);
-    const float rl = near ? lo : lo * scale * t.x;
-    const float b0 = near ? 0.0f : (float)e, b1 = near ? 0.0f : t.y, b2 = near ? 0.0f : t.z;
-    const float l2eh = 1.4426950216293335f, l2el = 1.925963033500011e-08f;   // log2(e) as a pair
-    // ln(1 + r + rl) = a + tail, the square split exactly, the cubic and the rest below 2^-23
-    const float q = r * r, qe = fmaf(r, r, -q);
-    float e0, e1, e2;
-    const float a = two_sum(r, -0.5f * q, &e0);
-    const float cub = q * r * (0.333333343f + r * (-0.25f + r * (0.2f + r * -0.166666672f)));
-    const float tail = (e0 - 0.5f * qe) + (fmaf(-r, rl, rl) + cub);
-    const float ph = a * l2eh;
-    const float pe = fmaf(tail, l2eh, fmaf(a, l2el, fmaf(a, l2eh, -ph)));
-    const float s1 = two_sum(b0, b1, &e1);
-    const float s2 = two_sum(s1, ph, &e2);
-    return make_float2(s2, ((e1 + e2) + b2) + pe);
-}
-
 // barrier of the NT computing threads (the potentials' warp takes no part)
 template <int NT>
 __device__ __forceinline__ void compute_sync() {

@@ -93,3 +93,17 @@ def test_resident_limits(ctx, steps, cap):
     u, v, info = api.sa_scale(ctx, d, ps, 1e-6, cap, kernel="step")
     assert info["steps_done"] == steps
     _check(ctx, w, d, ps, u, v, info, True)
+
+
+@pytest.mark.parametrize("kernel,n", [("step", 300), ("step", 3500), ("newton", 300)])
+def test_weights_up_to_2_31(ctx, kernel, n):
+    """int32 weights over their whole range, on both sides of the log2 table's line (2^15) and
+    beyond 24 bits, where a weight is a float and a remainder."""
+    rng = np.random.default_rng(44)
+    w = np.floor(2.0 ** rng.uniform(13.0, 31.0, (n, n))).astype(np.int64).clip(1, 2 ** 31 - 1).astype(np.int32)
+    w[:, :4] = [32767, 32768, 2 ** 24 + 1, 2 ** 31 - 1]
+    d = api.to_device(w)
+    ps = [1.0, 2.0, 4.0, 8.0]
+    u, v, info = api.sa_scale(ctx, d, ps, 1e-6, 20000, kernel=kernel)
+    assert info["status"] == 0, info
+    assert max(api.sa_verify(ctx, d, ps[-1], u, v)) < SUM_BOUND
