@@ -43,7 +43,7 @@ namespace sa {
 namespace {
 
 constexpr int kStepNred = 4;      // row-sum publication buffers
-constexpr int kStepMaxRps = 4;    // rows per ring stage at most
+constexpr int kStepMaxRps = 4;    // rows per ring stage that the scratch has room for (or RPS, if more)
 constexpr int kStepMaxRing = 16;  // ring slots at most; a slot holds one stage
 // rows per ring stage of the dense ring mode.  A stage costs a fixed ~0.5 us (the
 // publication of the warps' partial row sums and the slot's release) plus ~0.4 us per row
@@ -54,6 +54,12 @@ constexpr int kStepMaxRing = 16;  // ring slots at most; a slot holds one stage
 // two-stage ring consumes each stage before forming the next one's partials.
 constexpr int kDenseRowsPerStage = 2;
 constexpr int kWideRowsPerStage = 3;
+// For rows of 8 to 27 KB two slots of several row pairs: six rows while those fit (n <= 4492),
+// then four (n <= 6732); most n below 3300 are the resident kernel's.  Sweeps with four two-row slots (one stage ahead) and with these, us:
+// n = 3400 21.7 and 15.0, 4096 24.1 and 17.4, 4400 26.8 and 18.8; four rows 5000 29.6 and 22.6,
+// 6200 35.9 and 28.9.  Three slots of four rows: 16.1, 18.0 and 21.0 at the first three sizes, 17.8,
+// 19.8 and 22.8 when they also look one stage ahead.
+constexpr int kPairStages[] = {6, 4};
 
 struct StepArgs {
     const void* w;
@@ -178,8 +184,8 @@ struct KahanS {
     }
 };
 
-// SP: sparse epochs possible.  RPS: rows per ring stage (three for rows of 27 to 35 KB, one
-// for rows of more than 48 KB; two or three slots then).
+// SP: sparse epochs possible.  RPS: rows per ring stage (six or four for rows of 8 to 27 KB,
+// three for rows of 27 to 35 KB, one for rows of more than 48 KB; two or three slots then).
 template <int NT, int CH, bool SP, int RPS>
 __global__ void __launch_bounds__(NT, 1) step_kernel(StepArgs A) {
     constexpr int NW = NT / 32;
@@ -188,7 +194,7 @@ __global__ void __launch_bounds__(NT, 1) step_kernel(StepArgs A) {
     constexpr int MAXR = kStepMaxRing;
     constexpr int FG = NT / 64;
     static_assert(NT % 64 == 0, "layout");
-    static_assert(RPS >= 1 && RPS <= kStepMaxRps, "rows per stage");
+    constexpr int RED = RPS > kStepMaxRps ? RPS : kStepMaxRps;
     static_assert(!SP || RPS == 2, "sparse records come in stages of two rows");
     extern __shared__ __align__(128) unsigned char smem[];
     // [region: dense ring | or sparse c, S and ring] [barriers] [scratch]
@@ -199,7 +205,7 @@ __global__ void __launch_bounds__(NT, 1) step_kernel(StepArgs A) {
     unsigned* iss_cnt = rel_cnt + MAXR;                     // [MAXR] copies issued per slot
     // 8 (MAXR + NRED) + 8 MAXR bytes of barriers and counters end on a 16-byte boundary
     float* red = (float*)(iss_cnt + MAXR);                  // [NRED][RPS][NW] (16-aligned)
-    double* crow = (double*)(red + NRED * kStepMaxRps * NW);   // [max_rows] row references
+    double* crow = (double*)(red + NRED * RED * NW);   // [max_rows] row references
     double* redp = crow + A.max_rows;                       // [FG][64]
     double* redd = redp + FG * 64;                          // [NW]
     float* srow = (float*)(redd + NW);                      // [max_rows] row sums
@@ -696,10 +702,15 @@ __global__ void __launch_bounds__(NT, 1) step_kernel(StepArgs A) {
                         for (int r = 0; r < RPS; ++r)
                             if (r < nr) srow[q0 + r] = ss[r];
                     }
+                    // stages of several row pairs add them in the order two-row stages would
+                    constexpr bool kPairs = RPS > 2 && RPS % 2 == 0;
+                    const bool back = kPairs && ((v / (uint32_t)nst) & 1u) == 0u;
 #pragma unroll
-                    for (int r = 0; r < RPS; ++r) {
-                        if (r >= nr) break;
-                        const float inv = rcp_approx(ss[r]);
+                    for (int x = 0; x < RPS; ++x) {
+                        const int xb = kPairs ? (RPS - 2 - (x & ~1)) + (x & 1) : x;
+                        const int r = back ? xb : x;
+                        if (r >= nr) continue;
+                        const float inv = rcp_approx(back ? ss[xb] : ss[x]);
                         const unsigned char* rowp = row_of(v, q0, r);
                         if (SP && sparse) {
                             const uint2* rp = (const uint2*)rowp;
@@ -889,11 +900,11 @@ struct StepCfg {
     int rps;   // rows per ring stage
 };
 
-size_t step_smem_bytes(int nt, size_t region_bytes, int max_rows) {
+size_t step_smem_bytes(int nt, size_t region_bytes, int max_rows, int rps) {
     const int nw = nt / 32;
     const int fg = nt / 64;
     return region_bytes + 8 * (size_t)(kStepMaxRing + kStepNred) + 8 * (size_t)kStepMaxRing +
-           4 * (size_t)(kStepNred * kStepMaxRps * nw) +
+           4 * (size_t)(kStepNred * std::max(rps, kStepMaxRps) * nw) +
            8 * (size_t)(max_rows + fg * 64 + nw) + 4 * (size_t)max_rows + 8 * (size_t)max_rows + 4096 + 1024;
 }
 
@@ -920,11 +931,15 @@ StepCfg pick_step(const sa_ctx* ctx, int n) {
     const unsigned row_bytes = (unsigned)align_up((size_t)n * 4, 16);
     const int max_rows = step_max_rows(ctx, n);
     auto fits = [&](int ring) {
-        return step_smem_bytes(c.nt, (size_t)ring * row_bytes, max_rows) <= ctx->smem_optin;
+        return step_smem_bytes(c.nt, (size_t)ring * row_bytes, max_rows, c.rps) <= ctx->smem_optin;
+    };
+    auto fits_pairs = [&](int rows) {   // with the kernel's static shared memory
+        return step_smem_bytes(c.nt, 2 * (size_t)rows * row_bytes, max_rows, rows) + 4352 <= ctx->smem_optin;
     };
     // ring slots in rows, a whole number of stages, at least two: one-row stages for rows of
-    // 48 to 96 KB (two or three fit); else two-row stages, up to four, unless at most three
-    // of them fit and two three-row stages do.  The ring doubles as scratch for V
+    // 48 to 96 KB (two or three fit); two stages of six or four rows where n > 2048 and they
+    // fit; else two-row stages, up to four, unless at most three of them fit and two
+    // three-row stages do.  The ring doubles as scratch for V
     // (8 ceil(n/4)*4 bytes = two rows) during the per-step evaluation of K.
     if (c.rps == 1) {
         for (int st = 3; st >= 2; --st)
@@ -933,6 +948,12 @@ StepCfg pick_step(const sa_ctx* ctx, int n) {
                 return c;
             }
     } else {
+        for (const int rows : kPairStages)
+            if (!ctx->step_sparse && (c.ch == 2 || c.ch == 4) && fits_pairs(rows)) {
+                c.rps = rows;
+                c.ring = 2 * rows;
+                return c;
+            }
         int st2 = 0;
         for (int st = 4; st >= 2 && st2 == 0; --st)
             if (fits(st * kDenseRowsPerStage)) st2 = st;
@@ -1107,7 +1128,7 @@ sa_status scale_step(sa_ctx* ctx, const sa_matrix* a, const sa_scale_opts* o, do
     args.max_rows = step_max_rows(ctx, n);
     args.wait_ns = ctx->wait_ns;
     args.extra_arrivals = ctx->test_unreachable_barrier ? 1u : 0u;
-    const size_t smem = step_smem_bytes(cfg.nt, region, args.max_rows);
+    const size_t smem = step_smem_bytes(cfg.nt, region, args.max_rows, cfg.rps);
     int G = ctx->max_grid > 0 ? std::min(G_max, ctx->max_grid) : G_max;
     cudaEvent_t ev0, ev1;
     SA_CUDA(cudaEventCreate(&ev0));
@@ -1116,8 +1137,11 @@ sa_status scale_step(sa_ctx* ctx, const sa_matrix* a, const sa_scale_opts* o, do
     if (cfg.nt == 128) rc = launch_step<128, 1>(ctx, args, smem, &G);
     else if (cfg.nt == 256) rc = launch_step<256, 1>(ctx, args, smem, &G);
     else if (cfg.ch == 1) rc = launch_step<512, 1>(ctx, args, smem, &G);
+    else if (cfg.ch == 2 && cfg.rps == 6) rc = launch_step<512, 2, 6>(ctx, args, smem, &G);
     else if (cfg.ch == 2) rc = launch_step<512, 2>(ctx, args, smem, &G);
     else if (cfg.ch == 4 && cfg.rps == kWideRowsPerStage) rc = launch_step<512, 4, kWideRowsPerStage>(ctx, args, smem, &G);
+    else if (cfg.ch == 4 && cfg.rps == 6) rc = launch_step<512, 4, 6>(ctx, args, smem, &G);
+    else if (cfg.ch == 4 && cfg.rps == 4) rc = launch_step<512, 4, 4>(ctx, args, smem, &G);
     else if (cfg.ch == 4) rc = launch_step<512, 4>(ctx, args, smem, &G);
     else if (cfg.ch == 6 && cfg.rps == kWideRowsPerStage) rc = launch_step<512, 6, kWideRowsPerStage>(ctx, args, smem, &G);
     else if (cfg.ch == 6) rc = launch_step<512, 6>(ctx, args, smem, &G);
