@@ -18,8 +18,8 @@
 // exp(p log(w) - u - v) in FP64 rounds the logarithm, the product and both differences at
 // their magnitude: against extended precision the sums of n = 1000 matrices at p = 64 .. 512 are
 // off by 1e-16 to 1.2e-14 (relative, 2-norm), by 6e-15 to 2e-13 in that formula.  Potentials
-// that are not finite or leave F below 44 take that formula instead (mode 0), and so do
-// matrices below kVerifyFixedN, whose entries are too few to pay for the tables.
+// that are not finite or leave F below 44 take that formula instead (mode 0).  The tables pay at
+// every size: 59 - 75 us for a call with n = 8 .. 512 (int32), 61 - 171 us with mode 0.
 #include <algorithm>
 #include <cmath>
 
@@ -34,7 +34,6 @@ constexpr int kVerifyWarps = kVerifyThreads / 32;
 constexpr int kVerifyGroup = 8;                     // rows reduced together
 constexpr int kVerifyTab = 32768;                   // weights with a table entry of p log2 w
 constexpr int kExpTab = 4096;
-constexpr int kVerifyFixedN = 160;
 
 struct VerifyParams {
     int mode;        // 1: fixed point, 0: FP64 exp and log
@@ -64,7 +63,7 @@ struct VerifyView {
 
 // One block: the largest magnitude of the potentials and of p log2 w gives F.
 __global__ void __launch_bounds__(1024) verify_bounds_kernel(const double* u, const double* v, int n, double p, double log2w_max,
-                                     int allow_fixed, VerifyParams* par) {
+                                     VerifyParams* par) {
     __shared__ double sh[32];
     double m = p * log2w_max;
     int bad = 0;
@@ -79,7 +78,7 @@ __global__ void __launch_bounds__(1024) verify_bounds_kernel(const double* u, co
     if (threadIdx.x == 0) {
         for (int k = 1; k < (int)(blockDim.x >> 5); ++k) m = fmax(m, sh[k]);
         VerifyParams o{0, 0, 0, 0.0};
-        if (allow_fixed && !bad && m < 0x1p17) {
+        if (!bad && m < 0x1p17) {
             const int F = min(57, 61 - ilogb(m + 1.0) - 1);   // m < 2^(61 - F)
             o.F = F;
             o.mode = F >= 44;
@@ -308,10 +307,15 @@ sa_status verify_device(sa_ctx* ctx, const sa_matrix* a, double p, const double*
     const bool i16 = a->wtype == SA_I16;
     const int vec = 16 / wbytes(a->wtype);
     const int tiles = (n + 32 * vec - 1) / (32 * vec);
-    // rows a warp: about two waves of blocks, at least one group and at most 32 rows
+    // rows a warp: about two waves of blocks, at most 32 rows and at least one group, but n / 128
+    // for a small matrix, whose time is the chain of one lane's entries.  Whole calls at
+    // n = 8, 64, 256 and 1000 (us): 59, 61, 72 and 98 (int16), 59, 61, 72 and 84 (int32);
+    // 90, 95, 96 and 97, 83, 83, 88 and 87 with a group of eight rows.  With n / 256
+    // n = 1000 (int32) takes 98, with n / 64 n = 512 takes 98 and 86 instead of 84 and 75.
     const int want = std::max(1, 8 * ctx->num_sms / tiles);
     int rpw = (n + want * kVerifyWarps - 1) / (want * kVerifyWarps);
     rpw = std::min(32, std::max(kVerifyGroup, (int)align_up((size_t)rpw, kVerifyGroup)));
+    rpw = std::min(rpw, std::max(1, n / 128));
     const int chunks = (n + rpw * kVerifyWarps - 1) / (rpw * kVerifyWarps);
     const size_t need = 2 * align_up((size_t)n * 8, 256) + align_up((size_t)tiles * n * 8, 256) +
                         align_up((size_t)chunks * n * 8, 256) + 2 * (size_t)kVerifyTab * 8 + (size_t)kExpTab * 8 + 4096;
@@ -345,16 +349,13 @@ sa_status verify_device(sa_ctx* ctx, const sa_matrix* a, double p, const double*
     A.rpart = cv.take<double>((size_t)tiles * n);
     A.cpart = cv.take<double>((size_t)chunks * n);
     SA_CUDA(cudaMemsetAsync(mx, 0, 16, st));
-    verify_bounds_kernel<<<1, 1024, 0, st>>>(d_u, d_v, n, p, i16 ? 15.0 : 31.0, n >= kVerifyFixedN, par);
-    if (n >= kVerifyFixedN) {
-        verify_tables_kernel<<<kVerifyTab / 256, 256, 0, st>>>(d_u, d_v, n, p, par, Uf, Vf, T, R, E);
-        count_launch();
-    }
+    verify_bounds_kernel<<<1, 1024, 0, st>>>(d_u, d_v, n, p, i16 ? 15.0 : 31.0, par);
+    verify_tables_kernel<<<kVerifyTab / 256, 256, 0, st>>>(d_u, d_v, n, p, par, Uf, Vf, T, R, E);
     const dim3 g(tiles, chunks);
     if (i16) verify_kernel<int16_t><<<g, kVerifyThreads, 0, st>>>(A);
     else verify_kernel<int32_t><<<g, kVerifyThreads, 0, st>>>(A);
     verify_combine_kernel<<<dim3((n + 127) / 128, 2), 128, 0, st>>>(n, tiles, A.rpart, chunks, A.cpart, d_rows, d_cols, mx);
-    count_launch(3);
+    count_launch(4);
     SA_CUDA(cudaMemcpyAsync(ctx->pinned.ptr, mx, 16, cudaMemcpyDeviceToHost, st));
     SA_CUDA(cudaStreamSynchronize(st));
     SA_CUDA(cudaGetLastError());

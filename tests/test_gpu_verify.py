@@ -43,8 +43,11 @@ def _exact(w, p, u, v):
 
 
 @pytest.mark.parametrize("n,dtype,hi,p,scale,padded", [
-    (159, np.int16, 32767, 8.0, 1.0, True),        # below the fixed-point line
-    (160, np.int16, 32767, 1.0, 1.0, True),        # on it
+    (1, np.int32, 77, 8.0, 1.0, False),            # one entry
+    (7, np.int16, 32767, 64.0, 1.0, True),         # less than one tile of columns
+    (33, np.int32, 1 << 20, 16.0, 1.0, False),     # one row past a warp's lanes
+    (159, np.int16, 32767, 8.0, 1.0, True),
+    (160, np.int16, 32767, 1.0, 1.0, True),
     (257, np.int16, 30000, 64.0, 1.0, True),       # a tile and one column
     (513, np.int32, 1000, 256.0, 1.0, True),
     (255, np.int32, 2 ** 31 - 1, 3.7, 1.0, True),  # the largest weights, p with a full mantissa
