@@ -50,15 +50,14 @@ constexpr int kStepMaxRing = 16;  // ring slots at most; a slot holds one stage
 // at n = 8192, so two-row stages beat one-row stages (34.7 against 47.7 us per row pass)
 // although a one-row ring keeps twice the rows in flight.  Where at most three two-row
 // stages fit and two three-row stages do (rows of 27 to 35 KB), three-row stages are taken:
-// at n = 8192 45.5 against 48.0 us per sweep (row pass 33.7 against 37.1 us), although the
-// two-stage ring consumes each stage before forming the next one's partials.
+// at n = 8192 45.5 against 48.0 us per sweep (row pass 33.7 against 37.1 us).
 constexpr int kDenseRowsPerStage = 2;
 constexpr int kWideRowsPerStage = 3;
 // For rows of 8 to 27 KB two slots of several row pairs: six rows while those fit (n <= 4492),
-// then four (n <= 6732); most n below 3300 are the resident kernel's.  Sweeps with four two-row slots (one stage ahead) and with these, us:
-// n = 3400 21.7 and 15.0, 4096 24.1 and 17.4, 4400 26.8 and 18.8; four rows 5000 29.6 and 22.6,
-// 6200 35.9 and 28.9.  Three slots of four rows: 16.1, 18.0 and 21.0 at the first three sizes, 17.8,
-// 19.8 and 22.8 when they also look one stage ahead.
+// then four (n <= 6732); most n below 3300 are the resident kernel's.  Sweeps with four two-row
+// slots and with these, us: n = 3400 21.7 and 15.0, 4096 24.1 and 17.4, 4400 26.8 and 18.8; four rows
+// 5000 29.6 and 22.6, 6200 35.9 and 28.9.  Three slots of four rows: 16.1, 18.0 and 21.0 at the
+// first three sizes.
 constexpr int kPairStages[] = {6, 4};
 
 struct StepArgs {
@@ -735,14 +734,13 @@ __global__ void __launch_bounds__(NT, 1) step_kernel(StepArgs A) {
                     if (lane == 0) release_index(v);
                     return true;
                 };
-                // With three or more ring stages the partial row sums of stage g + 1 are
-                // formed while the other warps' partials of stage g are still arriving.  A
-                // two-stage ring cannot look ahead: the slot of g + 1 is refilled only when
-                // g + 1 - 2 is released, so each stage is consumed first and its copy for
-                // g + 2 is in flight while the next stage is read.  (Forming g + 1's partials
-                // first whenever its copy had already landed measured slower: 46.7 against
-                // 45.5 us per sweep at n = 8192 with three-row stages.)
-                if ((SP && sparse) || ring_n > 2) {
+                // A dense stage is consumed before the next one's partial row sums are formed, and its
+                // slot's refill is in flight meanwhile.  Forming the partials of stage g + 1 while
+                // the other warps' partials of g arrive holds a slot back for longer than that
+                // wait: 122.6 against 107.7 us a sweep at n = 12500, 138.6 and 122.1 at 14000, 182.2
+                // and 170.7 at 17000 (three slots), 8.9 and 7.6 at 256, 15.0 and 13.4 at 2000 (four).
+                // (Where the next copy had already landed only: 46.7 against 45.5 us at n = 8192.)
+                if (SP && sparse) {
                     if (nst > 0) produce(0);
                     for (int g = 0; g < nst; ++g) {
                         if (g + 1 < nst) produce(g + 1);
