@@ -11,8 +11,8 @@ grouped into size buckets and each bucket gets the shape that measured fastest f
   memory, 1, 2 or 4 groups per block (at most 8 warps per block);
 * the register path (n <= 128): K in registers during the sweeps, 1, 2 or 4 warps per
   instance up to n = 32, 4 or 8 up to 64, 16 up to 128 (at most 16 warps per block);
-* the K rows path: one block of 256 threads per instance on K kept in a global slot, each
-  warp on whole rows;
+* the K rows path: K of an instance in the registers and shared memory of one block (n <= 144)
+  or of a cluster of two or four, each warp on whole rows;
 * the block path: one block of 256 threads per instance, an SFU exp2 per term and sweep.
 
 :func:`tune` times every candidate of every bucket on a seeded synthetic pack of that

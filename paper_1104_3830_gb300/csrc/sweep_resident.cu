@@ -4,8 +4,8 @@
 // What bounds these sizes: the row pass of the streaming kernel reads K through a ring at
 // 0.7 us a stage and a sweep passes two grid barriers, so a sweep took 9.0 us at n = 256,
 // 11.7 us at n = 1000 and 16 us at n = 2047, of which arithmetic and L2 bytes are under 1 us.
-// Here a sweep takes 3.3, 4.4 and 7 us (whole calls with their evaluations of K: 4.20 -> 1.52 ms,
-// 5.40 -> 2.02 ms for 450 sweeps, 6.02 -> 2.77 ms for 360), most of it two exchanges between all blocks
+// Here a sweep takes 3.3, 4.4 and 6 us (whole calls with their evaluations of K: 4.20 -> 1.52 ms,
+// 5.40 -> 2.02 ms for 450 sweeps, 6.02 -> 2.46 ms for 360), most of it two exchanges between all blocks
 // through L2 (a store and the polls that find it, about 1 us each with the blocks of both
 // dies) and the chains of dependent instructions between them:
 //  * block b holds its row stripe of K: the first RR rows in registers (a thread owns 4 CH columns
