@@ -57,13 +57,13 @@ def load_peaks():
 # capture was taken on: after any change to these files the figure is unknown (null).
 _TRAFFIC = {
     # step kernel: planted n=8192 int16, p=256 from a cold start, 200 sweeps + 1 evaluation of K
-    (3, 8192, 2): ((37.355624e9 + 0.927293e9) / 200, "ncu capture, planted n=8192 int16, p=256, 200 sweeps (one launch)",
+    (3, 8192, 2): ((37.387707e9 + 0.926690e9) / 200, "ncu capture, planted n=8192 int16, p=256, 200 sweeps (one launch)",
                    {"paper_1104_3830_gb300/csrc/sweep_step.cu":
-                    "2714eb0a87182dc9e9501bed35d548eb3c7986a9c9daa6e21a14acfc754e8af6",
+                    "ec7cf3c035fdf124528b1da552c85b126f4083e26f21ea62ef9c524347fbbbd5",
                     "paper_1104_3830_gb300/csrc/common.cuh":
-                    "081ba7d34dae961c3679ac9acf1c076fd6b30bb4428eb03eabf3ad582049a6cc",
+                    "6a17ef3a88976f4542f96c1ff5adfadc1aea10906e7a2b68a8070b6884f59bb2",
                     "paper_1104_3830_gb300/csrc/log2pair.cuh":
-                    "d0d997e23dba7b51d1c07b556aa6d5e60d23cf230a79b17de392b2f3074ae3d0"}),
+                    "31cb7eff7990c018688083b63218d3f04f2e917126141686cdaf1e7fc079df2d"}),
     # step kernel: uniform n=20000 int16, the whole p = 1..256 schedule (28 sweeps, 9 evaluations
     # of K) of one scaling call, per sweep
     (3, 20000, 2): ((69.183675e9 + 17.738929e9) / 28,
