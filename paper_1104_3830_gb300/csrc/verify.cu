@@ -11,7 +11,7 @@
 // integer part of E (the exponent field), 12 bits (a 4096-entry table in shared memory) and
 // exp(t) - 1 = t + t^2 (1/2 + t/6), |t| < 2^-13, whose second part (below 2^-27) is formed in FP32.
 // Five FP64 instructions per entry are left (int16; nine for weights above 2^15), two of them
-// the sums: 0.89 ms at n = 8192 (0.57 ms of it those five at the FP64 rate).
+// the sums: 0.78 - 0.81 ms at n = 8192 (0.57 ms of it those five at the FP64 rate).
 //
 // Error: the fraction has F = 61 - ceil(log2 M) bits, M the largest of p log2 w, |U| and |V|, and
 // the table's logarithms are formed to 2^-57, so E is off by a few 2^-F, where
@@ -185,9 +185,13 @@ __device__ __forceinline__ double fixed_exp2(long long e, int F, const double* t
 // A warp owns a tile of 32 VEC columns (VEC = 16 bytes of weights a lane) and rows_per_warp rows;
 // the eight warps of a block take consecutive row chunks of one column tile, so that a block
 // writes one partial per column.  The row sums of eight rows are reduced together: each
-// exchange halves the rows that a lane still carries (9 additions instead of 40).
+// exchange halves the rows that a lane still carries (9 additions instead of 40).  Three blocks an
+// SM (80 registers; the int16 form spills 168 bytes) hide more of the FP64 latency than two: whole
+// calls at n = 5000, 8192 and 12000 take 372, 807 and 1580 us (int16), 547, 1323 and 2736 us
+// (int32), with two 384, 893 and 1718, 620, 1357 and 2807 us; n = 3000 (int16), whose last wave is
+// nearly empty then, 184 against 174 us.
 template <typename WT>
-__global__ void __launch_bounds__(kVerifyThreads) verify_kernel(VerifyView A) {
+__global__ void __launch_bounds__(kVerifyThreads, 3) verify_kernel(VerifyView A) {
     constexpr int VEC = 16 / sizeof(WT);
     __shared__ double tab[kExpTab];
     const VerifyParams P = *A.par;
