@@ -185,7 +185,8 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
     __shared__ float4 s_l2tab[256];
     __shared__ double s_ltab[256];
     __shared__ float s_red[kResMaxRows * NW];     // row partials of the warps
-    __shared__ float s_inv[kResMaxRows], s_sum[kResMaxRows];
+    __shared__ __align__(16) float s_inv[kResMaxRows];   // read four at a time
+    __shared__ float s_sum[kResMaxRows];
     __shared__ double s_cref[kResMaxRows], s_u[kResMaxRows];
     __shared__ unsigned s_rmax[kResMaxRows];
     __shared__ int s_fail, s_ok;
