@@ -413,7 +413,10 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
                 a0 = fmaf(kv.z, cf[4 * kk + 2], a0);
                 a1 = fmaf(kv.w, cf[4 * kk + 3], a1);
             };
-            auto reduce8 = [&](float s[8], int q0) {
+            // the sums of rows q0 .. q0 + 7 below `end`: a row's word is stored by the group that owns
+            // it alone (RR need not be a multiple of eight, and two lanes' stores to one word
+            // are not ordered)
+            auto reduce8 = [&](float s[8], int q0, int end) {
                 const bool b4 = lane & 16, b3 = lane & 8, b2 = lane & 4;
 #pragma unroll
                 for (int r = 0; r < 4; ++r) s[r] = (b4 ? s[r + 4] : s[r]) + __shfl_xor_sync(0xffffffffu, b4 ? s[r] : s[r + 4], 16);
@@ -423,7 +426,7 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
                 x += __shfl_xor_sync(0xffffffffu, x, 2);
                 x += __shfl_xor_sync(0xffffffffu, x, 1);
                 const int q = q0 + (lane >> 2);
-                if ((lane & 3) == 0 && q < kResMaxRows) s_red[q * NW + wid] = x;
+                if ((lane & 3) == 0 && q < end) s_red[q * NW + wid] = x;
             };
 #pragma unroll
             for (int g = 0; g < (RR + 7) / 8; ++g) {
@@ -440,7 +443,7 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
                     }
                     s[r] = a0 + a1;
                 }
-                reduce8(s, 8 * g);
+                reduce8(s, 8 * g, RR);
             }
             for (int q0 = RR; q0 < nrows; q0 += 8) {
                 float s[8];
@@ -453,7 +456,7 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
                         dot(ksm[(min(q0 + r, nrows - 1) - RR) * NC + min(cidx[kk], NC - 1)], kk, a0, a1);
                     s[r] = a0 + a1;
                 }
-                reduce8(s, q0);
+                reduce8(s, q0, nrows);
             }
             compute_sync<NT>();
             {

@@ -6,6 +6,7 @@ import numpy as np
 import pytest
 
 import oracle
+from paper_1104_3830_gb300 import _lib as L
 from paper_1104_3830_gb300 import api
 from paper_1104_3830_gb300 import workloads as W
 
@@ -107,3 +108,29 @@ def test_weights_up_to_2_31(ctx, kernel, n):
     u, v, info = api.sa_scale(ctx, d, ps, 1e-6, 20000, kernel=kernel)
     assert info["status"] == 0, info
     assert max(api.sa_verify(ctx, d, ps[-1], u, v)) < SUM_BOUND
+
+
+def _launches(call):
+    """The call's result and the kernels it launched: from a cold start the resident kernel
+    is one launch, the streaming kernel three (its potentials are converted afterwards)."""
+    n0 = L.lib().sa_kernel_launches()
+    r = call()
+    return r, L.lib().sa_kernel_launches() - n0
+
+
+# a form of each width with rows of the stripe in shared memory: 19 and 20 rows on 128 and 256
+# threads (16 in registers), 20 and 16 on 512 threads (14 in registers, so that the last group
+# of eight register rows is partly empty)
+@pytest.mark.parametrize("n,grid", [(300, 16), (1000, 52), (1300, 66), (2000, 126)])
+def test_resident_rows_in_shared_memory(ctx, n, grid):
+    w = W.uniform(n, 1, 1000, 45 + n, dtype=np.int16)
+    w[::3, 1::7] = 0
+    d = api.to_device(w)
+    ps = [1.0, 2.0, 4.0]
+    api.sa_set_option(ctx, "max_grid", grid)
+    try:
+        (u, v, info), k = _launches(lambda: api.sa_scale(ctx, d, ps, 1e-6, 20000, kernel="step"))
+    finally:
+        api.sa_set_option(ctx, "max_grid", 0)
+    assert k == 1
+    _check(ctx, w, d, ps, u, v, info, True)
