@@ -467,17 +467,18 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
                 }
                 s += __shfl_xor_sync(0xffffffffu, s, 1);
                 s += __shfl_xor_sync(0xffffffffu, s, 2);
+                bool in_range = true;
                 if (ox == 0 && oc < nrows) {
-                    if (!(s >= 0x1p-120f && s <= 0x1p120f)) {
-                        atomicCAS(A.err, 0, kErrNonfinite);
-                        s_fail = 1;
-                    }
+                    in_range = s >= 0x1p-120f && s <= 0x1p120f;
+                    if (!in_range) atomicCAS(A.err, 0, kErrNonfinite);
                     s_sum[oc] = s;
                     s_inv[oc] = rcp_approx(s);
                 }
+                // decided by the barrier itself: s_fail may already be set by a thread in the polls
+                // below while another has not read it here, and the threads that stay would wait for
+                // the one that left
+                if (!compute_sync_and<NT>(in_range)) return;
             }
-            compute_sync<NT>();
-            if (s_fail) return;
             // column partials c_j sum_q K_qj / s_q, the rows in the streaming kernel's order (pairs
             // of rows, last pair first in the first sweep of a step and in every other one after):
             // the same sums to the last bit whichever kernel a size takes

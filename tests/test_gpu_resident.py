@@ -134,3 +134,24 @@ def test_resident_rows_in_shared_memory(ctx, n, grid):
         api.sa_set_option(ctx, "max_grid", 0)
     assert k == 1
     _check(ctx, w, d, ps, u, v, info, True)
+
+
+@pytest.mark.parametrize("n", [300, 1300, 3000])
+def test_resident_row_sum_out_of_range_ends_every_block(ctx, n):
+    """A warm start whose potential of one row is far too large: that row of K underflows, its block
+    finds the sum out of range in the middle of a sweep and the others, waiting for its words, leave
+    on the error.  The warm start stays as given and the context usable."""
+    w = W.uniform(n, 1, 1000, 46, dtype=np.int16)
+    d = api.to_device(w)
+    ps = [1.0, 2.0]
+    u, v, _ = api.sa_scale(ctx, d, ps[:1], 1e-6, 20000, kernel="step")
+    for row in (0, n // 3, n - 1) * 3:
+        u1, v1 = u.clone(), v.clone()
+        u1[row] += 400.0
+        u0, v0 = u1.clone(), v1.clone()
+        with pytest.raises(api.SaError) as e:
+            api.sa_scale(ctx, d, ps, 1e-6, 20000, kernel="step", resume_from=1, u=u1, v=v1)
+        assert e.value.status == L.SA_E_NONFINITE, e.value
+        assert torch.equal(u1, u0) and torch.equal(v1, v0)
+    u, v, info = api.sa_scale(ctx, d, ps, 1e-6, 20000, kernel="step", resume_from=1, u=u, v=v)
+    _check(ctx, w, d, ps, u, v, info, n <= 1300)
