@@ -155,3 +155,27 @@ def test_resident_row_sum_out_of_range_ends_every_block(ctx, n):
         assert torch.equal(u1, u0) and torch.equal(v1, v0)
     u, v, info = api.sa_scale(ctx, d, ps, 1e-6, 20000, kernel="step", resume_from=1, u=u, v=v)
     _check(ctx, w, d, ps, u, v, info, n <= 1300)
+
+
+def test_resident_subnormal_column_sums(ctx):
+    """A column whose entries of K lie at 2^-125.6: in the first sweep its sum is 2^-126.9, below the
+    normal FP32 numbers, and its factor 2^126.9 is still finite.  Two sweeps against the same two in
+    FP64; FP32 keeps 19 bits of the column's terms, a wrong exponent would be off by 0.3 or more."""
+    n, p = 16, 6.28
+    w = np.full((n, n), 1 << 20, dtype=np.int32)
+    w[:, 0] = 0
+    w[:6, 0] = 1
+    u, v, info = api.sa_scale(ctx, api.to_device(w), [p], 1e-12, 2, kernel="step")
+    assert info["sweeps_total"] == 2, info
+    b = p * oracle.log_weights(w.astype(np.int64))
+    vo = np.zeros(n)
+    for _ in range(2):
+        uo = np.log(np.exp(b - vo - 80.0).sum(1)) + 80.0
+        vo = np.log(np.exp(b - uo[:, None]).sum(0))
+    assert np.max(np.abs(v.cpu().numpy() - vo)) < 1e-3
+    assert np.max(np.abs(u.cpu().numpy() - uo)) < 1e-3
+    # three entries: the sum is 2^-128 and the factor beyond 2^127 is cut, not infinite
+    w[3:6, 0] = 0
+    u, v, info = api.sa_scale(ctx, api.to_device(w), [p], 1e-12, 2, kernel="step")
+    assert info["status"] == L.SA_E_NOT_CONVERGED, info
+    assert torch.isfinite(u).all() and torch.isfinite(v).all()
