@@ -53,8 +53,8 @@ constexpr int kStepMaxRing = 16;  // ring slots at most; a slot holds one stage
 // at n = 8192 45.5 against 48.0 us per sweep (row pass 33.7 against 37.1 us).
 constexpr int kDenseRowsPerStage = 2;
 constexpr int kWideRowsPerStage = 3;
-// For rows of 8 to 27 KB two slots of several row pairs: six rows while those fit (n <= 4492),
-// then four (n <= 6732); most n below 3300 are the resident kernel's.  Sweeps with four two-row
+// For rows of 8 to 27 KB two slots of several row pairs: six rows while those fit (n <= 4508),
+// then four (n <= 6768); most n below 3300 are the resident kernel's.  Sweeps with four two-row
 // slots and with these, us: n = 3400 21.7 and 15.0, 4096 24.1 and 17.4, 4400 26.8 and 18.8; four rows
 // 5000 29.6 and 22.6, 6200 35.9 and 28.9.  Three slots of four rows: 16.1, 18.0 and 21.0 at the
 // first three sizes.
@@ -898,6 +898,9 @@ struct StepCfg {
     int rps;   // rows per ring stage
 };
 
+// static shared memory of every step_kernel (log2 table and flags; -Xptxas -v)
+constexpr size_t kStepStatic = 4224;
+
 size_t step_smem_bytes(int nt, size_t region_bytes, int max_rows, int rps) {
     const int nw = nt / 32;
     const int fg = nt / 64;
@@ -928,11 +931,11 @@ StepCfg pick_step(const sa_ctx* ctx, int n) {
     else return c;
     const unsigned row_bytes = (unsigned)align_up((size_t)n * 4, 16);
     const int max_rows = step_max_rows(ctx, n);
-    auto fits = [&](int ring) {
-        return step_smem_bytes(c.nt, (size_t)ring * row_bytes, max_rows, c.rps) <= ctx->smem_optin;
-    };
-    auto fits_pairs = [&](int rows) {   // with the kernel's static shared memory
-        return step_smem_bytes(c.nt, 2 * (size_t)rows * row_bytes, max_rows, rows) + 4352 <= ctx->smem_optin;
+    // a ring of `ring` rows in stages of `rps`, with the kernel's static shared memory.  The 5 KB
+    // that step_smem_bytes adds behind the arrays are spare: rings that need them were no better
+    // (n = 4604, six rows a stage 23.0, four 22.8 us a sweep; 18300, three slots 221, two 213)
+    auto fits = [&](int ring, int rps) {
+        return step_smem_bytes(c.nt, (size_t)ring * row_bytes, max_rows, rps) + kStepStatic <= ctx->smem_optin;
     };
     // ring slots in rows, a whole number of stages, at least two: one-row stages for rows of
     // 48 to 96 KB (two or three fit); two stages of six or four rows where n > 2048 and they
@@ -941,21 +944,21 @@ StepCfg pick_step(const sa_ctx* ctx, int n) {
     // (8 ceil(n/4)*4 bytes = two rows) during the per-step evaluation of K.
     if (c.rps == 1) {
         for (int st = 3; st >= 2; --st)
-            if (fits(st)) {
+            if (fits(st, 1)) {
                 c.ring = st;
                 return c;
             }
     } else {
         for (const int rows : kPairStages)
-            if (!ctx->step_sparse && (c.ch == 2 || c.ch == 4) && fits_pairs(rows)) {
+            if (!ctx->step_sparse && (c.ch == 2 || c.ch == 4) && fits(2 * rows, rows)) {
                 c.rps = rows;
                 c.ring = 2 * rows;
                 return c;
             }
         int st2 = 0;
         for (int st = 4; st >= 2 && st2 == 0; --st)
-            if (fits(st * kDenseRowsPerStage)) st2 = st;
-        if (st2 <= 3 && (c.ch == 4 || c.ch == 6) && fits(2 * kWideRowsPerStage)) {
+            if (fits(st * kDenseRowsPerStage, kDenseRowsPerStage)) st2 = st;
+        if (st2 <= 3 && (c.ch == 4 || c.ch == 6) && fits(2 * kWideRowsPerStage, kWideRowsPerStage)) {
             c.rps = kWideRowsPerStage;
             c.ring = 2 * kWideRowsPerStage;
             return c;

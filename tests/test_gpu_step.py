@@ -302,3 +302,15 @@ def test_far_steps_of_p(ctx):
     assert info["status"] == -4 and info["sweeps_total"] == 6, info
     er, ec = api.sa_verify(ctx, d, 256.0, u, v)
     assert ec < 1e-5 and np.isfinite(er)
+
+
+@pytest.mark.parametrize("n", [4604, 6765, 6900, 6920, 9009, 9188, 9220, 17921, 18276, 18340])
+def test_rings_that_fill_the_shared_memory(ctx, n):
+    """Sizes whose ring leaves little of an SM's shared memory beside the kernel's own arrays: the
+    default path takes every n up to 24576."""
+    w = W.uniform(n, 1, 1000, 970, dtype=np.int16)
+    d = api.to_device(w)
+    ps = [1.0, 2.0]
+    u, v, info = api.sa_scale(ctx, d, ps, 1e-6, 2000)
+    assert info["status"] == 0 and info["kernel_used"] == 3, info
+    assert max(api.sa_verify(ctx, d, ps[-1], u, v)) < STEP_SUM_BOUND
