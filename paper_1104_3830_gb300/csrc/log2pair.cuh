@@ -63,8 +63,9 @@ __device__ __forceinline__ float2 log2_pair(int w, const float4* tab) {
     return make_float2(s2, ((e1 + e2) + t.z) + small);
 }
 
-// log2 of s = hi + lo > 0 as a pair, to about 2^-46 (rms; 2^-43.7 at most): the reduction of sum_log2 in FP32 (m g - 1
-// is exact: 24 + 8 bits of which the leading 8 cancel)
+// log2 of s = hi + lo (hi a normal number) as a pair, to about 2^-46 of an exponent up to 31 (rms; 2^-43.6
+// at most): the reduction of sum_log2 in FP32 (m g - 1 is exact: 24 + 8 bits of which the
+// leading 8 cancel)
 __device__ __forceinline__ float2 pair_log2(float hi, float lo, const float4* tab) {
     const unsigned bits = __float_as_uint(hi);
     const int e = (int)(bits >> 23) - 127;
@@ -90,15 +91,50 @@ __device__ __forceinline__ float2 pair_log2(float hi, float lo, const float4* ta
     return make_float2(s2, ((e1 + b2) + pe) + e2);
 }
 
-// log2 of a positive integer weight as a float pair, from the shared table: the short series for
-// the int16 range, the longer one above it, where a weight is a float and an exact remainder.  (An
-// FP64 logarithm there took the first evaluation of K about 45 FP64 instructions an entry, at two
-// of them per clock and SM: 0.4 ms of 2.8 at n = 2047, and growing as n^2.)  Both carry log2 w at
-// least as closely as the pair's own second part does above the int16 range (2^-44).
-__device__ __forceinline__ float2 wlog2(const float4* stab, int w) {
-    if (w < kLog2Tab) return log2_pair(w, stab);
+// log2 of a weight of 2^15 .. 2^31 - 1 as a pair: pair_log2's reduction of the weight as a float and an
+// exact remainder (r exact, |r| < 2^-7.4; rl below 2^-24), every term kept to 2^-49 and
+// the pair normalised, so that only the rounding of its second part is left: rms 2^-46.2, at
+// most 2^-44.9 over 20 million weights, as an FP64 logarithm split into a pair.  Some thirty more FP32
+// instructions than pair_log2 (2^-43.6 at most), once an entry and call; the FP64 logarithm is about
+// 45 FP64 instructions, at two of them per clock and SM: 0.4 ms of 2.8 at n = 2047, growing as n^2.
+__device__ __forceinline__ float2 wide_log2(int w, const float4* tab) {
     const float hi = (float)w;                                   // up to 2^31
-    return pair_log2(hi, (float)(int)((unsigned)w - (unsigned)hi), stab);
+    const float lo = (float)(int)((unsigned)w - (unsigned)hi);
+    const unsigned bits = __float_as_uint(hi);
+    const int ex = (int)(bits >> 23) - 127;
+    const float4 t = tab[(bits >> 15) & 0xffu];
+    const float m = __uint_as_float((bits & 0x7fffffu) | 0x3f800000u);
+    const float r = fmaf(m, t.x, -1.0f);
+    const float rl = lo * __uint_as_float((unsigned)(127 - ex) << 23) * t.x;   // exact
+    const float l2eh = 1.4426950216293335f, l2el = 1.925963033500011e-08f;   // log2(e) as a pair
+    float e0, e1, e2, e3, e4, e5, e6, e7, ke;
+    const float q = __fmul_rn(r, r), qe = fmaf(r, r, -q);
+    const float a = two_sum(r, -0.5f * q, &e0);
+    // r^3 (1/3 - r/4 + r^2/5 - r^3/6) as a pair
+    const float c = __fmul_rn(q, r), ce = fmaf(qe, r, fmaf(q, r, -c));
+    const float k = two_sum(0.333333343f, __fmul_rn(r, fmaf(r, fmaf(r, -0.166666672f, 0.2f), -0.25f)), &ke);
+    ke -= 9.934108e-09f;                                         // 0.333333343f - 1/3
+    const float ch = __fmul_rn(c, k), cl = fmaf(ce, k, fmaf(c, ke, fmaf(c, k, -ch)));
+    // ln(1 + r + rl) = a + th + tl, with rl / (1 + r) - rl^2 / 2 for the remainder
+    const float th = two_sum(ch, rl, &e3);
+    const float tl = e3 + (cl + (e0 + fmaf(rl, q - (r + fmaf(0.5f, rl, c)), -0.5f * qe)));
+    const float ph = __fmul_rn(a, l2eh), pe = fmaf(a, l2eh, -ph);
+    const float xh = __fmul_rn(th, l2eh);
+    const float xl = fmaf(th, l2el, fmaf(tl, l2eh, fmaf(a, l2el, pe)) + fmaf(th, l2eh, -xh));
+    const float s1 = two_sum(t.y, ph, &e1);
+    const float s2 = two_sum((float)ex, s1, &e2);
+    float v = two_sum(e2, e1, &e4);
+    v = two_sum(v, t.z, &e5);
+    v = two_sum(v, xh, &e6);
+    v = two_sum(v, xl, &e7);
+    const float h = two_sum(s2, v, &e3);
+    return make_float2(h, e3 + (e7 + (e4 + (e5 + e6))));
+}
+
+// log2 of a positive integer weight as a float pair, from the shared table: the short series for
+// the int16 range, the longer one above it.
+__device__ __forceinline__ float2 wlog2(const float4* stab, int w) {
+    return w < kLog2Tab ? log2_pair(w, stab) : wide_log2(w, stab);
 }
 
 // 2^(p log2 w - V_j - m) with the operands as float pairs (p = ph + pl): the large leading
