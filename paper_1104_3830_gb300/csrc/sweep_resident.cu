@@ -189,7 +189,7 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
     __shared__ float s_sum[kResMaxRows];
     __shared__ double s_cref[kResMaxRows], s_u[kResMaxRows];
     __shared__ unsigned s_rmax[kResMaxRows];
-    __shared__ int s_fail, s_ok;
+    __shared__ int s_fail, s_range, s_ok;
     // between the owners and the potentials' warp, as (value, sweep number) words: the partial
     // sums of the columns and Vs - V, both as pairs; the decision (sweep number and done bit, by sweep parity)
     __shared__ uint4 s_S[CS * FG], s_D[kResMaxRows];
@@ -220,7 +220,7 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
     for (int j = tid; j < CS * FG; j += NT + 32) s_S[j] = make_uint4(0u, 0u, 0u, 0u);
     if (tid < kResMaxRows) s_D[tid] = make_uint4(0u, 0u, 0u, 0u);
     if (tid == 0) {
-        s_fail = 0;
+        s_fail = s_range = 0;
         s_dec[0] = s_dec[1] = 0u;
     }
     unsigned nbar = 1;
@@ -467,18 +467,20 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
                 }
                 s += __shfl_xor_sync(0xffffffffu, s, 1);
                 s += __shfl_xor_sync(0xffffffffu, s, 2);
-                bool in_range = true;
                 if (ox == 0 && oc < nrows) {
-                    in_range = s >= 0x1p-120f && s <= 0x1p120f;
-                    if (!in_range) atomicCAS(A.err, 0, kErrNonfinite);
+                    if (!(s >= 0x1p-120f && s <= 0x1p120f)) {
+                        atomicCAS(A.err, 0, kErrNonfinite);
+                        s_range = 1;
+                    }
                     s_sum[oc] = s;
                     s_inv[oc] = rcp_approx(s);
                 }
-                // decided by the barrier itself: s_fail may already be set by a thread in the polls
-                // below while another has not read it here, and the threads that stay would wait for
-                // the one that left
-                if (!compute_sync_and<NT>(in_range)) return;
             }
+            compute_sync<NT>();
+            // a flag that only the lines above set: s_fail may already be set by a thread in the polls
+            // below while another has not read it here, and the threads that stay would wait
+            // for the one that left
+            if (s_range) return;
             // column partials c_j sum_q K_qj / s_q, the rows in the streaming kernel's order (pairs
             // of rows, last pair first in the first sweep of a step and in every other one after):
             // the same sums to the last bit whichever kernel a size takes
