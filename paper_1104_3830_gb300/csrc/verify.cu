@@ -96,8 +96,8 @@ __device__ __forceinline__ long long fixed_product(double x, double y, double yl
     return llrint(ldexp(h, F)) + llrint(ldexp(l, F));
 }
 
-// log2 of k (0 < k < 2^15) with 58 fraction bits: the mantissa is squared, and each time it
-// passes 2 a bit of the logarithm is 1 (the errors of the truncated squares halve with
+// log2 of k (0 < k < 2^15) with 58 fraction bits, digit by digit: the mantissa is squared, and
+// each time it passes 2 a bit of the logarithm is 1 (the errors of the truncated squares halve with
 // every bit: below 2^-57 in all)
 __device__ unsigned long long log2_fixed58(unsigned k) {
     const int e = 31 - __clz(k);
@@ -151,16 +151,19 @@ __device__ __forceinline__ long long fixed_plog(const VerifyView& A, const Verif
     const int s = 17 - __clz(w);                       // w >> s in [2^14, 2^15)
     const int hi = w >> s;
     const unsigned lo = (unsigned)w & ((1u << s) - 1u);
-    const double lod = __hiloint2double(0x43300000, (int)lo) - 0x1p52;
+    // lo (below 2^17) in FP64 from its FP32 bits (0: 2^-127, which adds nothing)
+    const unsigned lb = __float_as_uint((float)(int)lo);
+    const double lod = __hiloint2double((int)(lb >> 3) + 0x38000000, (int)(lb << 29));
     const double r = __ldg(A.R + hi);
     const double d = lod * __hiloint2double(__double2hiint(r) - (s << 20), __double2loint(r));   // < 2^-14
-    // d in FP32 from its bits (0: lo = 0, else d is at least 2^-31)
+    // ln(1 + d) = (d - d^2 / 2) + d^3 (1/3 - d/4): the first part in FP64, the second, below 2^-43, in FP32
+    // (d cut to FP32 from its bits; 0: lo = 0, else d is at least 2^-31)
     const float df = lo ? __uint_as_float(((unsigned)(__double2hiint(d) - 0x38000000) << 3) | ((unsigned)__double2loint(d) >> 29)) : 0.0f;
-    const float q = df * df * (0.5f - df * (0.333333343f - 0.25f * df));   // d - ln(1 + d)
-    const unsigned qb = __float_as_uint(q);
-    const double qd = __hiloint2double((int)(qb >> 3) + 0x38000000, (int)(qb << 29));
+    const unsigned cb = __float_as_uint(df * df * df * (0.333333343f - 0.25f * df));
+    const double cd = __hiloint2double((int)(cb >> 3) + 0x38000000, (int)(cb << 29));
+    const double nh = __hiloint2double((int)((unsigned)(__double2hiint(d) - 0x100000) ^ 0x80000000u), __double2loint(d));   // -d/2
     // below 2^51: the sum with 1.5 2^52 holds the rounded integer in its low bits
-    const double m = fma(P.clog, d - qd, 0x1.8p52);
+    const double m = fma(P.clog, fma(d, nh, d) + cd, 0x1.8p52);
     return __ldg(A.T + hi) + (long long)s * P.pfix + (__double_as_longlong(m) - 0x4338000000000000ll);
 }
 
@@ -187,7 +190,7 @@ __device__ __forceinline__ double fixed_exp2(long long e, int F, const double* t
 // writes one partial per column.  The row sums of eight rows are reduced together: each
 // exchange halves the rows that a lane still carries (9 additions instead of 40).  Three blocks an
 // SM (80 registers; the int16 form spills 168 bytes) hide more of the FP64 latency than two: whole
-// calls at n = 5000, 8192 and 12000 take 372, 807 and 1580 us (int16), 547, 1323 and 2736 us
+// calls at n = 5000, 8192 and 12000 take 372, 807 and 1580 us (int16), 547, 1299 and 2736 us
 // (int32), with two 384, 893 and 1718, 620, 1357 and 2807 us; n = 3000 (int16), whose last wave is
 // nearly empty then, 184 against 174 us.
 template <typename WT>

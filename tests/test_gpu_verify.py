@@ -81,3 +81,27 @@ def test_verify_potentials_that_are_not_finite(ctx):
     assert float(rows[3]) == 0.0
     assert np.allclose(rows.cpu().numpy(), r.astype(float), rtol=1e-12)
     assert np.allclose(cols.cpu().numpy(), c.astype(float), rtol=1e-12)
+
+
+@pytest.mark.parametrize("p", [3.0, 512.0])
+def test_verify_weights_above_the_table(ctx, p):
+    """One entry a row and column, so that a sum is one term 2^E of a weight of 2^15 .. 2^31 - 1.  E is a
+    sum of numbers rounded to units of 2^-F (the table's, the series', U and V in two parts each: at
+    most 3 units), F as the kernel chooses it; 2^E adds a few roundings of 2^-53."""
+    n = 2000
+    rng = np.random.default_rng(12)
+    wv = np.floor(2.0 ** rng.uniform(15.0, 31.0, n)).astype(np.int64)
+    wv[:6] = [32768, 32769, 65535, 65536, 2 ** 31 - 1, 2 ** 30]
+    w = np.zeros((n, n), dtype=np.int32)
+    pi = rng.permutation(n)
+    w[np.arange(n), pi] = wv
+    v = rng.normal(0.0, 2.0, n)
+    u = p * np.log(wv) - v[pi] + rng.normal(0.0, 1.0, n)
+    _, _, rows, cols = api.sa_verify(ctx, api.to_device(w), p, torch.from_numpy(u).cuda(), torch.from_numpy(v).cuda(),
+                                     want_sums=True)
+    L = np.longdouble
+    x = np.exp(L(p) * np.log(wv.astype(L)) - u.astype(L) - v[pi].astype(L))
+    m = max(p * 31, np.abs(u).max() * 1.4427, np.abs(v).max() * 1.4427)
+    tol = 3 * 2.0 ** -(60 - int(np.floor(np.log2(m + 1)))) * np.log(2) + 6 * 2.0 ** -53
+    assert np.max(np.abs(rows.cpu().numpy() - x) / x) < tol
+    assert np.max(np.abs(cols.cpu().numpy()[pi] - x) / x) < tol
