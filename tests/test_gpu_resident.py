@@ -179,3 +179,31 @@ def test_resident_subnormal_column_sums(ctx):
     u, v, info = api.sa_scale(ctx, api.to_device(w), [p], 1e-12, 2, kernel="step")
     assert info["status"] == L.SA_E_NOT_CONVERGED, info
     assert torch.isfinite(u).all() and torch.isfinite(v).all()
+
+
+@pytest.mark.parametrize("n", [130, 600, 1500, 2500])
+def test_streaming_forms_below_the_resident_range(ctx, n):
+    """The streaming kernel at sizes the resident one usually takes (every width below 4096), reached by
+    a schedule longer than the resident kernel's 64 steps."""
+    w = W.uniform(n, 1, 1000, 47, dtype=np.int16)
+    d = api.to_device(w)
+    ps = [1.0 + 0.05 * k for k in range(65)]
+    (u, v, info), k = _launches(lambda: api.sa_scale(ctx, d, ps, 1e-6, 20000, kernel="step"))
+    assert k == 3 and info["steps_done"] == 65
+    _check(ctx, w, d, ps, u, v, info, False)
+    b = oracle.log_weights(w.astype(np.int64))
+    uo, vo, _, _, st = oracle.sinkhorn(b, ps[-1:], 1e-6, 20000)
+    assert st == 0
+    x, xo = (oracle.xmatrix(b, ps[-1], *uv) for uv in ((u.cpu().numpy(), v.cpu().numpy()), (uo, vo)))
+    assert np.all(np.abs(x - xo) <= 8e-6 * np.maximum(xo, 1.0 / n) + 1e-9)
+
+
+@pytest.mark.parametrize("n", [1, 300, 1216, 2047, 3333])
+def test_which_sizes_are_resident(ctx, n):
+    d = api.to_device(W.uniform(n, 1, 1000, 48, dtype=np.int16))
+    assert _launches(lambda: api.sa_scale(ctx, d, [1.0], 1e-6, 20000, kernel="step"))[1] == 1
+
+
+def test_which_sizes_are_streamed(ctx):
+    d = api.to_device(W.uniform(3501, 1, 1000, 48, dtype=np.int16))
+    assert _launches(lambda: api.sa_scale(ctx, d, [1.0], 1e-6, 20000, kernel="step"))[1] == 3

@@ -67,3 +67,29 @@ def test_option_values_are_checked(ctx):
         with pytest.raises(api.SaError) as e:
             api.sa_set_option(ctx, name, bad)
         assert e.value.status == -1
+
+
+def test_streaming_kernel_wait_limit_runs_out(ctx):
+    """The same on a size whose K is streamed (the one above is taken by the kernel that keeps K on the
+    chip), from a cold start and a warm one."""
+    n = 4000
+    w = W.uniform(n, 1, 1000, 4201, dtype=np.int16)
+    d = api.to_device(w)
+    ps = [1.0, 2.0]
+    u0 = torch.linspace(-3.0, 5.0, n, dtype=torch.float64, device="cuda")
+    v0 = torch.linspace(7.0, -1.0, n, dtype=torch.float64, device="cuda")
+    api.sa_set_option(ctx, "wait_limit_ns", 1_000_000)
+    api.sa_set_option(ctx, "test_unreachable_barrier", 1)
+    try:
+        for resume in (0, 1):
+            u1, v1 = u0.clone(), v0.clone()
+            with pytest.raises(api.SaError) as e:
+                api.sa_scale(ctx, d, ps, 1e-6, 2000, kernel="step", resume_from=resume, u=u1, v=v1)
+            assert e.value.status == -8 and "timed out" in str(e.value), e.value
+        assert torch.equal(u1, u0) and torch.equal(v1, v0)
+    finally:
+        api.sa_set_option(ctx, "test_unreachable_barrier", 0)
+        api.sa_set_option(ctx, "wait_limit_ns", 2_000_000_000)
+    u, v, info = api.sa_scale(ctx, d, ps, 1e-6, 2000, kernel="step")
+    assert info["status"] == 0 and info["kernel_used"] == 3, info
+    assert max(api.sa_verify(ctx, d, ps[-1], u, v)) < 2e-6
