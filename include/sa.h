@@ -249,6 +249,8 @@ sa_status sa_verify(sa_ctx* ctx, const sa_matrix* a, double p, const double* d_u
  *   out     filled with library-owned host arrays (sa_csr_free).
  *   log_ub  may be NULL; receives the approximate optimality certificate of Prop. aoc,
  *           (1/p) (sum_i max_j (p log w_ij - v_j) + sum_j v_j) >= log w_opt(A).
+ * sa_prune and sa_certify pass their host vectors through page-locked memory of the context,
+ * which its first call of a size allocates: keep a context for many calls.
  */
 sa_status sa_prune(sa_ctx* ctx, const sa_matrix* a, double p, const double* d_u,
                    const double* d_v, double t, int32_t guard, sa_csr* out, double* log_ub);

@@ -97,7 +97,7 @@ __device__ __forceinline__ float2 pair_log2(float hi, float lo, const float4* ta
 // most 2^-44.9 over 20 million weights, as an FP64 logarithm split into a pair.  Some thirty more FP32
 // instructions than pair_log2 (2^-43.6 at most), once an entry and call; the FP64 logarithm is about
 // 45 FP64 instructions, at two of them per clock and SM: 0.4 ms of 2.8 at n = 2047, growing as n^2.
-__device__ __forceinline__ float2 wide_log2(int w, const float4* tab) {
+static __device__ __noinline__ float2 wide_log2(int w, const float4* tab) {
     const float hi = (float)w;                                   // up to 2^31
     const float lo = (float)(int)((unsigned)w - (unsigned)hi);
     const unsigned bits = __float_as_uint(hi);

@@ -23,8 +23,10 @@
 // t + 1, sent after that block read its factors of t.
 //
 // Precision as in the streaming kernel: K in FP32 from the float-pair exponent, FP32
-// multiply-adds, compensated sums of the column partials over the blocks, FP64 potentials and
-// residual.
+// multiply-adds, compensated sums of the column partials over the blocks, FP64 potentials.  The
+// column total behind the next factor and the stop test is a pair of FP32 numbers (2^-47) where the
+// streaming kernel forms it in FP64 and rounds factor and residual to FP32 as well; errors
+// against 64 bits over the range are the streaming kernel's (3e-11 to 8e-10 of X(p), both).
 #include <algorithm>
 #include <cmath>
 
@@ -482,8 +484,8 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
             // for the one that left
             if (s_range) return;
             // column partials c_j sum_q K_qj / s_q, the rows in the streaming kernel's order (pairs
-            // of rows, last pair first in the first sweep of a step and in every other one after):
-            // the same sums to the last bit whichever kernel a size takes
+            // of rows, last pair first in the first sweep of a step and in every other one after), so
+            // that the kernels' FP32 sums round alike
             float S[M];
 #pragma unroll
             for (int m = 0; m < M; ++m) S[m] = 0.0f;

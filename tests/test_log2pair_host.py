@@ -21,7 +21,9 @@ HARNESS = """
 #include <cuda_runtime.h>
 #undef __device__
 #undef __forceinline__
-#define __device__ static
+#undef __noinline__
+#define __device__
+#define __noinline__
 #define __forceinline__ inline
 static unsigned __float_as_uint(float f) { unsigned u; memcpy(&u, &f, 4); return u; }
 static float __uint_as_float(unsigned u) { float f; memcpy(&f, &u, 4); return f; }
