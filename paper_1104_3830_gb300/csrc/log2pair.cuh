@@ -41,9 +41,9 @@ __device__ __forceinline__ float4 log2_tab_entry(int j) {
     return make_float4((float)g, th, (float)(t - (double)th), 0.0f);
 }
 
-// log2 w (0 < w < 2^15) as an unevaluated float pair, accurate to about 2^-40: with
+// log2 w (0 < w < 2^15) as an unevaluated float pair, accurate to about 2^-40 (2^-38.7 at most): with
 // w = 2^e m, m g_j is exact (15 + 9 significant bits), so r = m g_j - 1 is exact and
-// |r| < 2^-8; log2 w = e + (-log2 g_j) + log2(1 + r), the last from its series with the
+// |r| < 2^-7.4; log2 w = e + (-log2 g_j) + log2(1 + r), the last from its series with the
 // leading product r log2(e) split exactly.
 __device__ __forceinline__ float2 log2_pair(int w, const float4* tab) {
     const unsigned bits = __float_as_uint((float)w);
