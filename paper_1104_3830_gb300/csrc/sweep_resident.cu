@@ -614,22 +614,21 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
                         }
                         // the potentials' warp is done with the last sweep's sums once Vs - V is there
                         st_pair(s_S + col * FG + grp, raw_hi, raw_lo, t);
+                        const float2 lg = pair_log2(hi, lo, s_l2tab);
+                        const float x = two_sum(dh, -lg.x, &e);
+                        float c_new = ex2_approx(x + (e + (dl - lg.y)));
                         if (!(hi >= 0x1p-126f) || !(hi < INFINITY)) {
                             if (!(hi > 0.0f) || !(hi < INFINITY)) {
                                 atomicCAS(A.err, 0, kErrNonfinite);
                                 tag |= 2u;
                             } else {
-                                // a sum below the normal numbers is scaled for the logarithm, which reads the
-                                // exponent field; its factor may lie beyond 2^127 and is cut there (the
-                                // potentials do not use the factor: the next sweep makes up for it)
-                                hi *= 0x1p64f;
-                                lo *= 0x1p64f;
-                                dl += 64.0f - fmaxf(dh + 64.0f - lg2_approx(hi) - 127.0f, 0.0f);
+                                // a sum below the normal numbers, where pair_log2 finds no exponent: scaled, and
+                                // to the FP32 rounding of an exponent near 127; a factor beyond 2^127 is cut (the
+                                // potentials do not use it: the next sweep makes up for it)
+                                c_new = ex2_approx(fminf(dh + (dl + (64.0f - lg2_approx(hi * 0x1p64f))), 127.0f));
                             }
                         }
-                        const float2 lg = pair_log2(hi, lo, s_l2tab);
-                        const float x = two_sum(dh, -lg.x, &e);
-                        const uint64_t word = pack_word(ex2_approx(x + (e + (dl - lg.y))), tag);
+                        const uint64_t word = pack_word(c_new, tag);
                         for (int r = grp; r < kResCopies; r += FG) st_word(A.cw + (size_t)r * A.npad + c0 + col, word);
                     }
                 }
