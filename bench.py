@@ -57,13 +57,13 @@ def load_peaks():
 # capture was taken on: after any change to these files the figure is unknown (null).
 _TRAFFIC = {
     # step kernel: planted n=8192 int16, p=256 from a cold start, 200 sweeps + 1 evaluation of K
-    (3, 8192, 2): ((37.357089e9 + 0.924465e9) / 200, "ncu capture, planted n=8192 int16, p=256, 200 sweeps (one launch)",
+    (3, 8192, 2): ((37.374524e9 + 0.923506e9) / 200, "ncu capture, planted n=8192 int16, p=256, 200 sweeps (one launch)",
                    {"paper_1104_3830_gb300/csrc/sweep_step.cu":
-                    "7aa61e15494f04b1e1e9c77454865ba3388054550b82f3e1261db06e7582d58d",
+                    "b5605676c59ecfb90a3d06319896689bebe5619d4b872de572e0416635bd5c3a",
                     "paper_1104_3830_gb300/csrc/common.cuh":
                     "6a17ef3a88976f4542f96c1ff5adfadc1aea10906e7a2b68a8070b6884f59bb2",
                     "paper_1104_3830_gb300/csrc/log2pair.cuh":
-                    "f17c9e3a756c58961947b1941135889aeea2affc86c4992d3be9c56e509090b3"}),
+                    "14280663640b32c9aa82cd9ed737572016a1f293e265243783ad524f491f9e6e"}),
     # step kernel: uniform n=20000 int16, the whole p = 1..256 schedule (28 sweeps, 9 evaluations
     # of K) of one scaling call, per sweep
     (3, 20000, 2): ((69.183675e9 + 17.738929e9) / 28,

@@ -135,14 +135,13 @@ __device__ __forceinline__ void cluster_instances(const Args& A, float* slot) {
 #pragma unroll 1
             for (int c4 = lane; c4 < NC; c4 += 32) {
                 const WT* wr = wb + (int64_t)(r0 + q) * ld + 4 * c4;
-                float2 x[4];
+                int w[4];
+                float lh[4], ll[4];
 #pragma unroll
-                for (int e = 0; e < 4; ++e) {
-                    const int w = 4 * c4 + e < n ? (int)wr[e] : 0;
-                    x[e] = w > 0 ? wlog2(sm.l2tab, w) : make_float2(-INFINITY, 0.0f);
-                }
-                *(float4*)(Lh + (int64_t)(r0 + q) * ldk + 4 * c4) = make_float4(x[0].x, x[1].x, x[2].x, x[3].x);
-                *(float4*)(Ll + (int64_t)(r0 + q) * ldk + 4 * c4) = make_float4(x[0].y, x[1].y, x[2].y, x[3].y);
+                for (int e = 0; e < 4; ++e) w[e] = 4 * c4 + e < n ? (int)wr[e] : 0;
+                wlog2_4(sm.l2tab, w, lh, ll);
+                *(float4*)(Lh + (int64_t)(r0 + q) * ldk + 4 * c4) = make_float4(lh[0], lh[1], lh[2], lh[3]);
+                *(float4*)(Ll + (int64_t)(r0 + q) * ldk + 4 * c4) = make_float4(ll[0], ll[1], ll[2], ll[3]);
             }
         float Kr[RG][M];
         int sweeps_all = 0;

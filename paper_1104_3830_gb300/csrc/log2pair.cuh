@@ -91,13 +91,20 @@ __device__ __forceinline__ float2 pair_log2(float hi, float lo, const float4* ta
     return make_float2(s2, ((e1 + b2) + pe) + e2);
 }
 
+// the same for |a| >= |b|
+__device__ __forceinline__ float fast_two_sum(float a, float b, float* err) {
+    const float s = a + b;
+    *err = b - (s - a);
+    return s;
+}
+
 // log2 of a weight of 2^15 .. 2^31 - 1 as a pair: pair_log2's reduction of the weight as a float and an
 // exact remainder (r exact, |r| < 2^-7.4; rl below 2^-24), every term kept to 2^-49 and
 // the pair normalised, so that only the rounding of its second part is left: rms 2^-46.2, at
-// most 2^-44.9 over 20 million weights, as an FP64 logarithm split into a pair.  Some thirty more FP32
-// instructions than pair_log2 (2^-43.6 at most), once an entry and call; the FP64 logarithm is about
-// 45 FP64 instructions, at two of them per clock and SM: 0.4 ms of 2.8 at n = 2047, growing as n^2.
-static __device__ __noinline__ float2 wide_log2(int w, const float4* tab) {
+// most 2^-44.96 over 20 million weights (an FP64 logarithm split into a pair 2^-44.91, pair_log2
+// 2^-43.6).  About 80 FP32 instructions; the FP64 logarithm is about 45 FP64 instructions, at two
+// of them per clock and SM: 0.4 ms of 2.8 at n = 2047, growing as n^2.
+__device__ __forceinline__ float2 wide_log2(int w, const float4* tab) {
     const float hi = (float)w;                                   // up to 2^31
     const float lo = (float)(int)((unsigned)w - (unsigned)hi);
     const unsigned bits = __float_as_uint(hi);
@@ -107,14 +114,14 @@ static __device__ __noinline__ float2 wide_log2(int w, const float4* tab) {
     const float r = fmaf(m, t.x, -1.0f);
     const float rl = lo * __uint_as_float((unsigned)(127 - ex) << 23) * t.x;   // exact
     const float l2eh = 1.4426950216293335f, l2el = 1.925963033500011e-08f;   // log2(e) as a pair
-    float e0, e1, e2, e3, e4, e5, e6, e7, ke;
+    const float th3 = 0.333333343f, tl3 = -9.934108e-09f;                      // 1/3 as a pair
+    float e1, e2, e3, e4;
+    // r - r^2 / 2 = a + e0 - qe / 2; r^3 (1/3 + s) = ch + cl
     const float q = __fmul_rn(r, r), qe = fmaf(r, r, -q);
-    const float a = two_sum(r, -0.5f * q, &e0);
-    // r^3 (1/3 - r/4 + r^2/5 - r^3/6) as a pair
+    const float a = fmaf(-0.5f, q, r), e0 = fmaf(-0.5f, q, r - a);
     const float c = __fmul_rn(q, r), ce = fmaf(qe, r, fmaf(q, r, -c));
-    const float k = two_sum(0.333333343f, __fmul_rn(r, fmaf(r, fmaf(r, -0.166666672f, 0.2f), -0.25f)), &ke);
-    ke -= 9.934108e-09f;                                         // 0.333333343f - 1/3
-    const float ch = __fmul_rn(c, k), cl = fmaf(ce, k, fmaf(c, ke, fmaf(c, k, -ch)));
+    const float s = r * fmaf(r, fmaf(r, -0.166666672f, 0.2f), -0.25f);
+    const float ch = __fmul_rn(c, th3), cl = fmaf(c, s, fmaf(ce, th3, fmaf(c, tl3, fmaf(c, th3, -ch))));
     // ln(1 + r + rl) = a + th + tl, with rl / (1 + r) - rl^2 / 2 for the remainder
     const float th = two_sum(ch, rl, &e3);
     const float tl = e3 + (cl + (e0 + fmaf(rl, q - (r + fmaf(0.5f, rl, c)), -0.5f * qe)));
@@ -122,19 +129,47 @@ static __device__ __noinline__ float2 wide_log2(int w, const float4* tab) {
     const float xh = __fmul_rn(th, l2eh);
     const float xl = fmaf(th, l2el, fmaf(tl, l2eh, fmaf(a, l2el, pe)) + fmaf(th, l2eh, -xh));
     const float s1 = two_sum(t.y, ph, &e1);
-    const float s2 = two_sum((float)ex, s1, &e2);
-    float v = two_sum(e2, e1, &e4);
-    v = two_sum(v, t.z, &e5);
-    v = two_sum(v, xh, &e6);
-    v = two_sum(v, xl, &e7);
-    const float h = two_sum(s2, v, &e3);
-    return make_float2(h, e3 + (e7 + (e4 + (e5 + e6))));
+    const float s2 = fast_two_sum((float)ex, s1, &e2);
+    float z = two_sum(e1, xh, &e3);
+    z = two_sum(z, t.z, &e4);
+    float zl = xl + (e3 + e4);
+    const float v = two_sum(e2, z, &e3);
+    zl += e3;
+    const float v2 = v + zl;
+    const float h = fast_two_sum(s2, v2, &e4);
+    return make_float2(h, e4 + ((v - v2) + zl));
 }
+// out of line: inlined in the unrolled loops over a row it made the evaluation longer for all
+// weights (n = 20000, int16: 1.86 against 1.75 ms)
+static __device__ __noinline__ float2 wide_log2_call(int w, const float4* tab) { return wide_log2(w, tab); }
 
 // log2 of a positive integer weight as a float pair, from the shared table: the short series for
 // the int16 range, the longer one above it.
 __device__ __forceinline__ float2 wlog2(const float4* stab, int w) {
-    return w < kLog2Tab ? log2_pair(w, stab) : wide_log2(w, stab);
+    return w < kLog2Tab ? log2_pair(w, stab) : wide_log2_call(w, stab);
+}
+
+// The same for four weights (-inf, 0 for one that is not positive): the four chains of a
+// wide logarithm overlap, and one call serves them.
+struct WideLog4 {
+    float4 h, l;
+};
+static __device__ __noinline__ WideLog4 wide_log4(int w0, int w1, int w2, int w3, const float4* tab) {
+    const float2 a = wide_log2(w0, tab), b = wide_log2(w1, tab), c = wide_log2(w2, tab), d = wide_log2(w3, tab);
+    return {make_float4(a.x, b.x, c.x, d.x), make_float4(a.y, b.y, c.y, d.y)};
+}
+__device__ __forceinline__ void wlog2_4(const float4* stab, const int w[4], float lh[4], float ll[4]) {
+    WideLog4 x{};
+    const bool wide = max(max(w[0], w[1]), max(w[2], w[3])) >= kLog2Tab;
+    if (wide) x = wide_log4(w[0], w[1], w[2], w[3], stab);
+    const float xh[4] = {x.h.x, x.h.y, x.h.z, x.h.w}, xl[4] = {x.l.x, x.l.y, x.l.z, x.l.w};
+#pragma unroll
+    for (int e = 0; e < 4; ++e) {
+        float2 p = make_float2(-INFINITY, 0.0f);
+        if (w[e] > 0) p = w[e] < kLog2Tab ? log2_pair(w[e], stab) : make_float2(xh[e], xl[e]);
+        lh[e] = p.x;
+        ll[e] = p.y;
+    }
 }
 
 // 2^(p log2 w - V_j - m) with the operands as float pairs (p = ph + pl): the large leading

@@ -316,12 +316,7 @@ __global__ void __launch_bounds__(NT + 32, 1) resident_kernel(const __grid_const
                 if (fresh) {
                     int wv[4];
                     res_load4(A, r0 + q, cidx[kk] * 4, nval[kk], wv);
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        const float2 l = wv[e] > 0 ? wlog2(s_l2tab, wv[e]) : make_float2(-INFINITY, 0.0f);
-                        lh[e] = l.x;
-                        ll[e] = l.y;
-                    }
+                    wlog2_4(s_l2tab, wv, lh, ll);
                     *(float4*)(A.Lh + at) = make_float4(lh[0], lh[1], lh[2], lh[3]);
                     *(float4*)(A.Ll + at) = make_float4(ll[0], ll[1], ll[2], ll[3]);
                 } else {

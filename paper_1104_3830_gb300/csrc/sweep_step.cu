@@ -448,16 +448,7 @@ __global__ void __launch_bounds__(NT, 1) step_kernel(StepArgs A) {
                 // log2 w of the chunk's entries as float pairs (-inf: no entry)
                 float lh[4], ll[4];
                 if constexpr (FRESH) {
-#pragma unroll
-                    for (int e = 0; e < 4; ++e) {
-                        lh[e] = -INFINITY;
-                        ll[e] = 0.0f;
-                        if (e < nval[k] && wv[4 * k + e] > 0) {
-                            const float2 lw = wlog2(s_l2tab, wv[4 * k + e]);
-                            lh[e] = lw.x;
-                            ll[e] = lw.y;
-                        }
-                    }
+                    wlog2_4(s_l2tab, wv + 4 * k, lh, ll);   // zeros beyond the row
                     if (cidx[k] < NC) {
                         *(float4*)(A.Lh + row * A.ldk + cidx[k] * 4) = make_float4(lh[0], lh[1], lh[2], lh[3]);
                         *(float4*)(A.Ll + row * A.ldk + cidx[k] * 4) = make_float4(ll[0], ll[1], ll[2], ll[3]);
