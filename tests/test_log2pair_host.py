@@ -46,6 +46,12 @@ extern "C" void weights_log2(const int* w, int n, float* hi, float* lo) {
         const float2 l = sa::wlog2(tab, w[k]);
         hi[k] = l.x;
         lo[k] = l.y;
+        if (k % 4 == 3) {   // four at a time: the same numbers
+            float h4[4], l4[4];
+            sa::wlog2_4(tab, w + k - 3, h4, l4);
+            for (int e = 0; e < 4; ++e)
+                if (h4[e] != hi[k - 3 + e] || l4[e] != lo[k - 3 + e]) hi[k - 3 + e] = NAN;
+        }
     }
 }
 """
@@ -79,7 +85,10 @@ def test_weights_above_the_int16_range(lib):
     # the ends of the range, and weights whose pair is hard to round
     w = np.concatenate([w, np.arange(32768, 98304), np.arange(2 ** 31 - 65536, 2 ** 31), 2 ** np.arange(15, 31),
                         [18263941, 71320028, 17170369, 460273136, 134730888]]).astype(np.int32)
+    w[::7] >>= 12   # some small neighbours, whose own logarithms are not what is bounded here
     e = _errors(lib, w)
+    assert np.all(np.isfinite(e))
+    e = e[w >= 32768]
     assert np.max(np.abs(e)) <= 2.0 ** -44.9
     assert np.sqrt(np.mean(e * e)) <= 2.0 ** -46.2
-    assert abs(np.mean(e)) <= 2.0 ** -46.2 / np.sqrt(len(w)) * 5   # no bias
+    assert abs(np.mean(e)) <= 2.0 ** -46.2 / np.sqrt(len(e)) * 5   # no bias
