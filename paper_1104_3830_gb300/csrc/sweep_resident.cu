@@ -26,7 +26,7 @@
 // multiply-adds, compensated sums of the column partials over the blocks, FP64 potentials.  The
 // column total behind the next factor and the stop test is a pair of FP32 numbers (2^-47) where the
 // streaming kernel forms it in FP64 and rounds factor and residual to FP32 as well; errors
-// against 64 bits over the range are the streaming kernel's (3e-11 to 8e-10 of X(p), both).
+// against 64 bits over the range are the streaming kernel's (3e-11 to 1e-9, both).
 #include <algorithm>
 #include <cmath>
 
